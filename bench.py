@@ -227,7 +227,7 @@ def pair_flops(m: int, n: int, D: int, shared: bool = False) -> dict:
 
 
 def modp_mults(m: int, n: int, D: int, primes: int) -> int:
-    """32-bit integer multiplies of the exact prefix path (radic_modp_prefix.cu)
+    """32-bit integer multiplies of the exact per-minor terms (radic_modp_prefix.cu)
     for all C(n,m) minors: a fraction-free update (a_kk a_ij - a_ik a_kj,
     Montgomery-reduced) is 4 multiplies, a Montgomery product 3, a reduction
     2, a leaf dot product (D = 3) 7.  Per prefix and prime: the elimination of
@@ -247,6 +247,22 @@ def modp_mults(m: int, n: int, D: int, primes: int) -> int:
         k = n - 1 - v
         tot += cnt * (per_pre + k * per_col + math.comb(k, 2) * per_pair + math.comb(k, D) * per_leaf)
     return tot * primes
+
+
+def modp_subtree_mults(m: int, n: int, G: int, primes: int) -> int:
+    """32-bit integer multiplies of the exact subtree sums (radic_modp_subtree.cuh) over all C(n,m)
+    minors: every product of residues is one multiply and every Montgomery reduction two.  Per head
+    of H = m-G columns and prime, at its j-th column: the m-j entries of the column (sums of j+1
+    products, unreduced products for j = 0), two products per updated coefficient; per later column
+    G entries (sums of H+1 products) and for every set of k >= 2 of the G rows a sum of k products;
+    per head the denominators (2H + G - 3 products) and the fraction update (3 products)."""
+    H = m - G
+    dot = lambda k: k + 2
+    head = 3 * (2 * H + G - 3) + 3 * 3
+    for j in range(1, H):
+        head += (m - j) * dot(j + 1) + (m - j - 1) * (j * dot(2) + dot(1))
+    col = G * dot(H + 1) + sum(math.comb(G, k) * dot(k) for k in range(2, G + 1))
+    return primes * sum(math.comb(v, H - 1) * (head + (n - 1 - v) * col) for v in range(H - 1, n - G))
 
 
 # ---------------------------------------------------------------------------
@@ -720,12 +736,12 @@ def measure_configs(R, W, torch, np, stream, flush, peaks, mats, A, minors, gold
     ms = ev_time(lambda: R.radic_det(a, mode="exact", out=res, workspace=ws), reps=3)
     r = R.parse_result(res)
     pinfo = R.radic_plan_info(12, 40, "exact")
-    mults = modp_mults(12, 40, pinfo["prefix_depth"], r["n_primes"])
+    mults = modp_subtree_mults(12, 40, pinfo["subtree_depth"], r["n_primes"])
     mult_rate = mults / (ms / 1e3) / 1e12
     out["int8_12x40_exact"] = {
         "value": r["minors"] / (ms / 1e3), "unit": UNIT, "ms": ms, "n_primes": r["n_primes"],
         "exact_ok": r["exact"] == int(golden_fraction("int8_12x40")),
-        "mapping": f"{pinfo['mapping']} depth {pinfo['prefix_depth']}",
+        "mapping": f"{pinfo['mapping']}, subtrees of {pinfo['subtree_depth']} columns",
         "roofline": {"bound": "alu", "achieved": mult_rate, "unit": "T multiplies/s",
                      "peak": peaks["int32_mad_wide_tops"] if peaks else None,
                      "frac": mult_rate / peaks["int32_mad_wide_tops"] if peaks else None,
@@ -741,7 +757,7 @@ def measure_configs(R, W, torch, np, stream, flush, peaks, mats, A, minors, gold
         "value": math.comb(32, 8) / (ms / 1e3), "unit": UNIT, "ms": ms, "n_primes": wr["n_primes"],
         "bits": abs(wr["integer"]).bit_length(),
         "exact_ok": wr["value_exact"] == golden_fraction("fp64_8x32"),
-        "what": "radic_det_exact_wide: RADIC_MAX_PRIMES primes per pass of the exact kernels, Garner to limbs"}
+        "what": "radic_det_exact_wide: every prime in one launch of the exact kernel, Garner to limbs in its last block"}
 
     # differentiation 256 x 6 x 28: forward (batched binary64) and backward
     Dm = torch.from_numpy(W.diff_256x6x28()).cuda()

@@ -105,7 +105,11 @@ enum { RADIC_MODE_FP64 = 0, RADIC_MODE_MIXED = 1, RADIC_MODE_EXACT = 2, RADIC_MO
  *            prefix's lexicographic subtree then costs one D x D
  *            determinant of Schur-complement entries (for D = 3 a scalar
  *            triple product).  Same pivots and elimination steps as
- *            per-minor LU, shared by the subtree.
+ *            per-minor LU, shared by the subtree.  In EXACT mode the
+ *            determinant needs only the signed sum, so the units are heads
+ *            of m-G columns (G = 2..6, from the plan's cost model, or an
+ *            explicit prefix_depth) whose subtrees are summed by linearity
+ *            without forming the minors; radic_terms uses depth D.
  *  AUTO   -- PREFIX when 3 <= m <= n within its limit, else THREAD when
  *            m <= 8 (12 for EXACT), else GROUP. */
 enum { RADIC_MAP_AUTO = 0, RADIC_MAP_THREAD = 1, RADIC_MAP_GROUP = 2, RADIC_MAP_PREFIX = 3 };
@@ -127,7 +131,9 @@ typedef struct radic_options {
                                3 (0: 3 when m >= 7 and n - m <= 3.5m, else 2) */
   int32_t lanes_per_prefix; /* PREFIX mapping: lanes of a warp that share the
                                leaves of one prefix (1, 2, 4, ..., 32; 0:
-                               per prefix group, from the plan's cost model) */
+                               per prefix group, from the plan's cost model;
+                               EXACT determinants, which form no leaves,
+                               always use the cost model)                    */
   int32_t deterministic;    /* PREFIX mapping, floating-point modes: 0
                                (default) = after its first task a warp draws
                                the next from a counter, which evens out the
@@ -212,15 +218,17 @@ size_t radic_workspace_bytes(int m, int n, int mode, const radic_options* opts);
  * depth (0 unless PREFIX), [2] group width (0 unless GROUP), [3] threads per
  * block, [4] blocks of the main kernel, [5] ranks per processor run (THREAD,
  * GROUP) or warp tasks (PREFIX), [6] dynamic shared memory bytes of the main
- * kernel, [7] workspace bytes.  Same errors as radic_det's planning. */
-#define RADIC_PLAN_INFO_COUNT 8
+ * kernel, [7] workspace bytes, [8] columns G of the summed subtrees (EXACT
+ * mode, PREFIX; 0 otherwise; [4] is then the blocks per prime).  Same errors
+ * as radic_det's planning. */
+#define RADIC_PLAN_INFO_COUNT 9
 int radic_plan_info(int m, int n, int mode, const radic_options* opts, int64_t* info, int count);
 
 /* Host-only view of the prefix mapping's task table (the Section 5 split of
  * the minors into contiguous runs, here runs of prefixes grouped by their
  * last column v), planned for `sms` SMs with `blocks_per_sm` resident blocks
  * instead of the current device: no GPU is touched.  opts->mapping is taken
- * as RADIC_MAP_PREFIX.  info (host, count >= 8 + 4n int64): [0] prefix depth
+ * as RADIC_MAP_PREFIX.  EXACT mode: the table of radic_terms.  info (host, count >= 8 + 4n int64): [0] prefix depth
  * D, [1] warp tasks, [2] blocks, [3] v_lo, [4] v_hi, [5] 1 when warps draw
  * tasks from the counter, [6..7] 0; then for every v four entries at
  * 8 + 4v: prefixes whose last column is v (C(v, m-D-1)), prefixes per lane
@@ -254,10 +262,11 @@ int radic_det(const void* A, int m, int n, int64_t lda, int dtype, int mode,
  * (integer inputs, and binary32/binary64 inputs as the dyadic rationals
  * they are), with as many 31-bit primes as the Hadamard bound of the scaled
  * integer rows needs, up to RADIC_WIDE_MAX_PRIMES (about 990 bits).  The
- * primes are taken RADIC_MAX_PRIMES per pass of the EXACT kernels (passes
- * whose primes the bound does not need return at once), and a last kernel
- * rebuilds the integer by mixed-radix (Garner) reconstruction into base-2^32
- * limbs.  Not a computation of the paper: its extension of the exact mode to
+ * integer is rebuilt by mixed-radix (Garner) reconstruction into base-2^32
+ * limbs.  PREFIX mapping: one launch serves every prime and its last block
+ * reconstructs; the per-minor mappings take RADIC_MAX_PRIMES primes per pass
+ * (passes whose primes the bound does not need return at once) and a last
+ * kernel reconstructs.  Not a computation of the paper: its extension of the exact mode to
  * inputs whose value does not fit 128 bits.
  * A: device, row-major m x n, leading dimension lda; out: device;
  * workspace: device, 256-byte aligned, radic_wide_workspace_bytes(m, n,

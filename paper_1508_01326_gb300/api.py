@@ -65,7 +65,7 @@ def radic_workspace_bytes(m: int, n: int, mode="fp64", options=None) -> int:
 
 
 PLAN_INFO_KEYS = ["mapping", "prefix_depth", "group_width", "threads", "blocks", "run_or_tasks", "smem_bytes",
-                  "workspace_bytes"]
+                  "workspace_bytes", "subtree_depth"]
 MAPPING_NAMES = {1: "thread", 2: "group", 3: "prefix"}
 
 

@@ -26,6 +26,8 @@ SOURCES = [
     "radic_pair.cu",
     "radic_modp.cu",
     "radic_modp_prefix.cu",
+    "radic_modp_subtree_lo.cu",
+    "radic_modp_subtree_hi.cu",
     "radic_noalloc.cu",
     "radic_batched.cu",
     "radic_batched_k32.cu",

@@ -1,6 +1,7 @@
 // C-ABI entry points of the single-matrix path: argument validation, launch
 // planning (mapping, grid, workspace layout) and launches.  Validation happens
 // entirely on the host before anything is enqueued.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -41,7 +42,7 @@ int blocks_per_sm(const SinglePlan& p) {
     case kModeFp64: return blocks_per_sm_fp64(p);
     case kModeMixed: return blocks_per_sm_mixed(p);
     case kModePair: return blocks_per_sm_pair(p);
-    default: return blocks_per_sm_modp(p);
+    default: return blocks_per_sm_modp(p, p.mapping == RADIC_MAP_PREFIX ? kModpTerms : kModpDet);
   }
 }
 
@@ -50,12 +51,97 @@ size_t smem_of(const SinglePlan& p) {
     case kModeFp64: return smem_fp64(p);
     case kModeMixed: return smem_mixed(p);
     case kModePair: return smem_pair(p);
-    default: return smem_modp(p);
+    default: return smem_modp(p, p.mapping == RADIC_MAP_PREFIX ? kModpTerms : kModpDet);
   }
 }
 
 void layout_workspace(SinglePlan& pl);
 
+// Cost of one head of H = m - G columns with k later columns in the subtree
+// kernel, in issued instructions: a dot product of N residues takes about
+// 1.4 N + 8 (multiply-adds at half rate, folds, reduction and correction).
+double subtree_cost(int m, int G, int k) {
+  const int H = m - G;
+  double head = 60.0, col = 0.0;
+  for (int j = 0; j < H; ++j) head += (m - j) * (1.4 * (j + 1) + 8.0) + (m - j - 1) * (11.0 * j + 6.0);
+  col += G * (1.4 * (H + 1) + 10.0);
+  for (int s = 1; s <= G; ++s) col += (double)binom_host(G, s) * (s == 1 ? 3.0 : 1.4 * s + 10.0);
+  return head + k * col;
+}
+
+// Subtree table of the EXACT determinant for heads of m - G columns: group v
+// (last head column) holds C(v, H-1) heads, one head per lane and task (or
+// ranks_per_task consecutive ones).  Heads with split_from or more later
+// columns take two lanes, each half of the columns.
+PrefixTable subtree_table(int m, int n, int G, int run_given, int split_from) {
+  const int H = m - G;
+  PrefixTable t{};
+  t.v_lo = H - 1;
+  t.v_hi = n - 1 - G;
+  unsigned long long start = 0;
+  for (int v = t.v_lo; v <= t.v_hi; ++v) {
+    t.count[v] = binom_host(v, H - 1);
+    t.lanes[v] = n - 1 - v >= split_from ? 2 : 1;
+    const unsigned long long groups = 32 / t.lanes[v];
+    t.run[v] = std::min<unsigned long long>(run_given > 0 ? run_given : 1, (t.count[v] + groups - 1) / groups);
+    t.task_start[v] = start;
+    start += (t.count[v] + groups * t.run[v] - 1) / (groups * t.run[v]);
+  }
+  if (t.v_hi + 1 < kMaxN) t.task_start[t.v_hi + 1] = start;
+  t.total_tasks = start;
+  return t;
+}
+
+// Depth G of the summed subtrees and from how many columns on a head takes two
+// lanes: an explicit prefix depth is taken as it is; otherwise the choice whose
+// estimated time is least.  Warps that share a scheduler issue about one of
+// these instructions in two cycles, a warp on its own one in six (measured on
+// the longest heads of 8 x 32): the estimate adds the work of the expected
+// primes spread over the chip's schedulers and the longest task alone.  Small
+// matrices thus take shallow subtrees (more, shorter lanes), large ones deep
+// subtrees; splitting the columns of the longest heads, whose groups are too
+// small to fill their warps anyway, nearly halves the longest task.  Every
+// block stages the matrix for its prime (5 to 9 us), so the blocks of the
+// expected primes together fill the chip once; large matrices take more
+// blocks, of at least eight tasks a warp, because the number of primes is only
+// known on the device and a last wave that is partly empty costs more.
+void plan_subtree(SinglePlan& pl, const radic_options& d, int sms) {
+  const int m = pl.m, n = pl.n;
+  for (int w = 0; w < 2; ++w) {
+    const double primes = w ? 12.0 : 2.0;  // typical counts: random binary64 rows; small integers
+    int best = 0;
+    double best_time = 0.0;
+    for (int G = 2; G <= kSubtreeMax && G < m; ++G) {
+      if (d.prefix_depth != 0 && G != d.prefix_depth) continue;
+      const int kmax = n - m + G;  // later columns of the longest head
+      for (const int split : {kMaxN + 1, (3 * kmax + 3) / 4, (kmax + 1) / 2}) {
+        const PrefixTable t = subtree_table(m, n, G, d.ranks_per_task, split);
+        double work = 0.0, longest = 0.0;
+        for (int v = t.v_lo; v <= t.v_hi; ++v) {
+          const int k = n - 1 - v;
+          const double c = (double)t.run[v] * (t.lanes[v] == 2 ? subtree_cost(m, G, (k + 1) / 2) + 4.0 * (1 << G)
+                                                                : subtree_cost(m, G, k));
+          const unsigned long long next = v < t.v_hi ? t.task_start[v + 1] : t.total_tasks;
+          work += c * (double)(next - t.task_start[v]);
+          longest = std::max(longest, c);
+        }
+        const double time = 2.0 * primes * work / (4.0 * sms) + 6.0 * longest;
+        if (best == 0 || time < best_time) {
+          best = G;
+          best_time = time;
+          pl.stab[w] = t;
+        }
+      }
+    }
+    pl.subtree[w] = best;
+    const int warps = pl.threads / 32;
+    const unsigned long long need = (pl.stab[w].total_tasks + warps - 1) / warps;
+    const int per_sm = std::max(1, blocks_per_sm_modp(pl, w ? kModpWide : kModpDet));
+    const unsigned long long fill = (unsigned long long)(sms * per_sm / primes) + 1;
+    const unsigned long long cap = std::max(fill, std::min(need / 8, 4ull * sms * per_sm));
+    pl.sub_blocks[w] = d.blocks > 0 ? d.blocks : (int)std::max(1ull, std::min(need, cap));
+  }
+}
 
 int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsigned long long units,
                 SinglePlan* out) {
@@ -127,6 +213,7 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
   pl.ranks_per_task = (units + procs - 1) / procs;
   if (pl.ranks_per_task < 1) pl.ranks_per_task = 1;
   pl.tasks = (units + pl.ranks_per_task - 1) / pl.ranks_per_task;
+  if (pl.mode == kModeExact) plan_subtree(pl, d, sms);
   layout_workspace(pl);
   *out = pl;
   return RADIC_OK;
@@ -258,7 +345,7 @@ int make_plan_uncached(int m, int n, int mode, const radic_options* o, unsigned 
 void layout_workspace(SinglePlan& pl) {
   const int mode = pl.mode;
   const int n_warps = pl.blocks * pl.threads / 32;
-  size_t off = 256;
+  size_t off = mode == kModeExact ? kExactHeaderBytes : kHeaderBytes;
   pl.off_partials = off;
   off = align_up(off + (size_t)pl.blocks * sizeof(FpPartial), 256);
   if (mode == kModeMixed || mode == kModePair) {
@@ -422,10 +509,14 @@ int radic_plan_info(int m, int n, int mode, const radic_options* opts, int64_t* 
   v[1] = (p.mapping == RADIC_MAP_PREFIX) ? p.depth : 0;
   v[2] = (p.mapping == RADIC_MAP_GROUP) ? p.group : 0;
   v[3] = p.threads;
-  v[4] = p.blocks;
-  v[5] = (p.mapping == RADIC_MAP_PREFIX) ? (int64_t)p.ptab.total_tasks : (int64_t)p.ranks_per_task;
-  v[6] = (int64_t)p.smem;
+  const bool subtree = p.mapping == RADIC_MAP_PREFIX && mode == kModeExact;
+  v[4] = subtree ? p.sub_blocks[0] : p.blocks;
+  v[5] = subtree                             ? (int64_t)p.stab[0].total_tasks
+         : (p.mapping == RADIC_MAP_PREFIX) ? (int64_t)p.ptab.total_tasks
+                                             : (int64_t)p.ranks_per_task;
+  v[6] = subtree ? (int64_t)smem_modp(p, kModpDet) : (int64_t)p.smem;
   v[7] = (int64_t)p.ws_bytes;
+  v[8] = subtree ? p.subtree[0] : 0;
   for (int i = 0; i < count; ++i) info[i] = v[i];
   return RADIC_OK;
 }
@@ -473,7 +564,8 @@ int radic_det(const void* A, int m, int n, int64_t lda, int dtype, int mode, con
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < p.ws_bytes)
     return RADIC_EWORKSPACE;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  if (cudaMemsetAsync(ws, 0, 256, s) != cudaSuccess) return RADIC_ECUDA;
+  if (cudaMemsetAsync(ws, 0, mode == kModeExact ? kExactHeaderBytes : kHeaderBytes, s) != cudaSuccess)
+    return RADIC_ECUDA;
   SingleArgs a;
   std::memset(&a, 0, sizeof(a));
   a.A = A;
@@ -494,6 +586,7 @@ int radic_det(const void* A, int m, int n, int64_t lda, int dtype, int mode, con
   a.flag_count = reinterpret_cast<int*>(ws + p.off_flag_count);
   a.flag_ranks = reinterpret_cast<unsigned long long*>(ws + p.off_flag_ranks);
   a.modp_partials = reinterpret_cast<uint32_t*>(ws + p.off_modp);
+  a.residue_sums = reinterpret_cast<unsigned long long*>(ws + kHeaderBytes);
   a.out = out;
   int r;
   switch (mode) {
@@ -528,8 +621,11 @@ int radic_det_exact_wide(const void* A, int m, int n, int64_t lda, int dtype, co
     return RADIC_EWORKSPACE;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   uint32_t* wide = reinterpret_cast<uint32_t*>(ws + off_wide);
-  for (int base = 0; base < kWidePrimes; base += kMaxPrimes) {
-    if (cudaMemsetAsync(ws, 0, 256, s) != cudaSuccess) return RADIC_ECUDA;
+  // the prefix mapping takes every prime in one launch and reconstructs in its
+  // last block; the per-minor mappings take RADIC_MAX_PRIMES per pass
+  const bool subtree = p.mapping == RADIC_MAP_PREFIX;
+  for (int base = 0; base < kWidePrimes; base += subtree ? kWidePrimes : kMaxPrimes) {
+    if (cudaMemsetAsync(ws, 0, kExactHeaderBytes, s) != cudaSuccess) return RADIC_ECUDA;
     SingleArgs a;
     std::memset(&a, 0, sizeof(a));
     a.A = A;
@@ -546,9 +642,12 @@ int radic_det_exact_wide(const void* A, int m, int n, int64_t lda, int dtype, co
     a.modp_partials = reinterpret_cast<uint32_t*>(ws + p.off_modp);
     a.prime_base = base;
     a.wide = wide;
+    a.residue_sums = reinterpret_cast<unsigned long long*>(ws + kHeaderBytes);
+    if (subtree) a.wide_out = out;
     const int r = launch_modp(p, a, s);
     if (r != RADIC_OK) return r;
   }
+  if (subtree) return RADIC_OK;
   return launch_wide_crt(wide, out, p.total, s);
 }
 

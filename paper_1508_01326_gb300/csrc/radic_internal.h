@@ -99,6 +99,11 @@ struct SinglePlan {
   int group = 0;                   // lanes per minor for the group mapping
   PrefixTable ptab{};              // prefix mapping only
   int depth = 2;                   // prefix mapping: trailing columns per leaf
+  // EXACT prefix mapping, determinant: heads of m - subtree columns; blocks
+  // per prime.  [0] radic_det, [1] the wide entry point (more primes)
+  PrefixTable stab[2]{};
+  int subtree[2] = {0, 0};
+  int sub_blocks[2] = {1, 1};
   int threads = 128;
   int blocks = 1;
   unsigned long long ranks_per_task = 64;
@@ -133,6 +138,8 @@ struct SingleArgs {
   uint32_t* modp_partials;  // blocks x kMaxPrimes residues
   int prime_base;           // EXACT: first prime of this pass (wide entry point; 0 otherwise)
   uint32_t* wide;           // EXACT wide passes: residues by prime index, then needed, exponent, status
+  unsigned long long* residue_sums;  // EXACT subtree kernel: per prime, zeroed before the call
+  radic_wide_result* wide_out;       // EXACT subtree kernel: wide result instead of `out`
   radic_result* out;
   // terms mode
   unsigned long long q0, count;
@@ -141,6 +148,11 @@ struct SingleArgs {
 
 unsigned long long binom_host(int n, int k);  // exact C(n, k) for n <= 64 (0 if k > n)
 int device_sm_count();
+
+// Bytes at the start of a workspace that are zeroed before a call: the header,
+// and in EXACT mode the residue sums of the subtree kernel after it.
+constexpr size_t kHeaderBytes = 256;
+constexpr size_t kExactHeaderBytes = kHeaderBytes + kWidePrimes * sizeof(unsigned long long);
 
 // Launchers (return a RADIC_* code).  When `args.terms` is non-null the
 // kernel writes per-rank terms instead of reducing.
@@ -153,15 +165,18 @@ int launch_wide_crt(const uint32_t* wide, radic_wide_result* out, unsigned long 
 int launch_unrank(int n, int m, unsigned long long q0, unsigned long long count, uint8_t* cols,
                   int ranks_per_task, cudaStream_t s);
 
+// What an EXACT kernel is planned for: radic_det, the wide entry point, terms.
+enum : int { kModpDet = 0, kModpWide = 1, kModpTerms = 2 };
+
 // Occupancy helpers filled in by the arithmetic files.
 int blocks_per_sm_fp64(const SinglePlan& p);
 int blocks_per_sm_mixed(const SinglePlan& p);
 int blocks_per_sm_pair(const SinglePlan& p);
-int blocks_per_sm_modp(const SinglePlan& p);
+int blocks_per_sm_modp(const SinglePlan& p, int use);
 size_t smem_fp64(const SinglePlan& p);
 size_t smem_mixed(const SinglePlan& p);
 size_t smem_pair(const SinglePlan& p);
-size_t smem_modp(const SinglePlan& p);
+size_t smem_modp(const SinglePlan& p, int use);
 
 // Persistent batched kernels per m and task path (argument: the batched
 // path's BatchArgs): binary32 tier, pair tier (m >= 3), binary64 tier;
@@ -170,9 +185,14 @@ const void* batch_kernel_f32(int m, int path);
 const void* batch_kernel_pair(int m, int path);
 const void* batch_kernel_f64(int m, int path);
 
-// Prefix kernel of the EXACT mode for (m, depth) (arguments: SingleArgs,
-// PrefixTable), or nullptr.
-const void* modp_prefix_kernel(int m, int depth, bool terms);
+// Prefix kernels of the EXACT mode (arguments: SingleArgs, PrefixTable), or
+// nullptr: per-minor terms for (m, depth); subtree sums for heads of m - G
+// columns, and their shared memory.
+const void* modp_prefix_kernel(int m, int depth);
+const void* modp_subtree_kernel(int m, int G);
+const void* modp_subtree_kernel_hi(int m, int G);  // m >= 9
+size_t modp_subtree_smem(int m, int n);
+constexpr int kSubtreeMax = 6;  // largest G (the sums hold 2^G - 1 registers)
 
 // Binary64 fix-up kernel of the MIXED and PAIR modes (arguments: SingleArgs,
 // int main_blocks, int tier) and its dynamic shared memory.

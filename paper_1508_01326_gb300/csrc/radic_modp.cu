@@ -14,9 +14,9 @@
 // unimodular matrix T = L U.  Every minor of T A has the same determinant as
 // the minor of A (det T = 1), and the rare zero pivot that remains takes a
 // slow path with row exchanges.  The group mapping chooses a nonzero pivot
-// row by ballot and needs no slow path.  The prefix mapping shares the
-// elimination of each (m-D)-column prefix among the minors of its subtree,
-// as the floating-point prefix kernels do, in non-dividing modular form.
+// row by ballot and needs no slow path.  The prefix mapping (its own files)
+// shares the elimination of a head of leading columns among the minors of its
+// subtree, in non-dividing modular form.
 #include "radic_modp.cuh"
 
 namespace radic {
@@ -211,8 +211,10 @@ const void* group_kernel(bool terms) {
                : reinterpret_cast<const void*>(&k_modp_group<G, false>);
 }
 
-const void* pick(const SinglePlan& p, bool terms) {
-  if (p.mapping == RADIC_MAP_PREFIX) return modp_prefix_kernel(p.m, p.depth, terms);
+const void* pick(const SinglePlan& p, int use) {
+  const bool terms = use == kModpTerms;
+  if (p.mapping == RADIC_MAP_PREFIX)
+    return terms ? modp_prefix_kernel(p.m, p.depth) : modp_subtree_kernel(p.m, p.subtree[use]);
   if (p.mapping == RADIC_MAP_THREAD) {
     switch (p.m) {
       case 1: return thread_kernel<1>(terms);
@@ -237,92 +239,30 @@ const void* pick(const SinglePlan& p, bool terms) {
 
 }  // namespace
 
-size_t smem_modp(const SinglePlan& p) {
+// Shared memory of the determinant kernel (terms: of the per-term kernel).
+size_t smem_modp(const SinglePlan& p, int use) {
+  if (p.mapping == RADIC_MAP_PREFIX && use != kModpTerms) return modp_subtree_smem(p.m, p.n);
   const int cs = (p.mapping != RADIC_MAP_GROUP) ? ((p.m + 3) / 4) * 4 : p.m;
   size_t b = modp_smem_bytes(p.n, p.m, cs, p.threads);
   if (p.mapping == RADIC_MAP_PREFIX) b += zbuf_bytes(p.n - p.m + p.depth, p.threads, p.depth, 4);
   return b;
 }
 
-int blocks_per_sm_modp(const SinglePlan& p) {
-  const void* k = pick(p, false);
+int blocks_per_sm_modp(const SinglePlan& p, int use) {
+  const void* k = pick(p, use);
   if (!k) return 0;
-  if (!allow_smem(k, smem_modp(p))) return 0;
+  const size_t smem = smem_modp(p, use);
+  if (!allow_smem(k, smem)) return 0;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, p.threads, smem_modp(p)) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, p.threads, smem) != cudaSuccess) return 0;
   return nb;
 }
 
-// ---------------------------------------------------------------------------
-// Wide exact result: mixed-radix (Garner) reconstruction of the integer from
-// its residues modulo the first K primes, then base-2^32 limbs by Horner's
-// rule over the mixed-radix digits, the symmetric range (-M/2, M/2) for the
-// sign, M the product of the primes.  One thread; K <= 32.
-// ---------------------------------------------------------------------------
-__device__ void limbs_mul_add(uint32_t* x, int nl, uint32_t mul, uint32_t add) {
-  uint64_t carry = add;
-  for (int i = 0; i < nl; ++i) {
-    const uint64_t t = static_cast<uint64_t>(x[i]) * mul + carry;
-    x[i] = static_cast<uint32_t>(t);
-    carry = t >> 32;
-  }
-}
-
 __global__ void k_wide_crt(const uint32_t* wide, radic_wide_result* out, unsigned long long total) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  constexpr int NL = RADIC_WIDE_LIMBS + 1;  // one spare limb for M
   const int needed = static_cast<int>(wide[kWidePrimes]);
-  const int escale = static_cast<int>(wide[kWidePrimes + 1]);
-  const int status = static_cast<int>(wide[kWidePrimes + 2]);
-  const int K = needed < kWidePrimes ? needed : kWidePrimes;
-  uint64_t v[kWidePrimes];
-  for (int i = 0; i < K; ++i) {
-    const uint64_t p = prime_at(i);
-    uint64_t acc = 0, prod = 1;  // digits so far and prod_{l<i} p_l, modulo p
-    for (int l = 0; l < i; ++l) {
-      acc = (acc + v[l] * prod) % p;
-      prod = (prod * (prime_at(l) % p)) % p;
-    }
-    const uint64_t diff = (wide[i] + p - acc) % p;
-    v[i] = (diff * powmod64(prod, p - 2, p)) % p;
-  }
-  uint32_t x[NL], mm[NL];
-  for (int i = 0; i < NL; ++i) x[i] = mm[i] = 0u;
-  mm[0] = 1u;
-  for (int i = K - 1; i >= 0; --i) limbs_mul_add(x, NL, prime_at(i), static_cast<uint32_t>(v[i]));
-  for (int i = 0; i < K; ++i) limbs_mul_add(mm, NL, prime_at(i), 0u);
-  // d = M - x; the value is x when x < d (that is x < M/2), else -(M - x)
-  uint32_t d[NL];
-  long long borrow = 0;
-  for (int i = 0; i < NL; ++i) {
-    const long long t = static_cast<long long>(mm[i]) - x[i] - borrow;
-    d[i] = static_cast<uint32_t>(t);
-    borrow = t < 0 ? 1 : 0;
-  }
-  bool x_less = false;
-  for (int i = NL - 1; i >= 0; --i) {
-    if (x[i] != d[i]) {
-      x_less = x[i] < d[i];
-      break;
-    }
-  }
-  const uint32_t* mag = x_less ? x : d;
-  int nl = 0;
-  for (int i = 0; i < RADIC_WIDE_LIMBS; ++i)
-    if (mag[i]) nl = i + 1;
-  for (int i = 0; i < RADIC_WIDE_LIMBS; ++i) out->limbs[i] = mag[i];
-  double val = 0.0;
-  const int lo = nl > 3 ? nl - 3 : 0;
-  for (int i = nl - 1; i >= lo; --i) val = val * 4294967296.0 + static_cast<double>(mag[i]);
-  const int sgn = nl == 0 ? 0 : (x_less ? 1 : -1);
-  out->value = sgn < 0 ? -ldexp(val, 32 * lo + escale) : ldexp(val, 32 * lo + escale);
-  out->status = (needed > kWidePrimes) ? RADIC_EOVERFLOW : status;
-  out->n_primes = K;
-  out->exact_exp = escale;
-  out->sign = sgn;
-  out->n_limbs = nl;
-  out->minors = static_cast<long long>(total);
-  out->reserved = 0;
+  const int K = min(needed, kWidePrimes);
+  wide_crt_warp((int)threadIdx.x < K ? wide[threadIdx.x] : 0u, K, needed, static_cast<int>(wide[kWidePrimes + 1]),
+                static_cast<int>(wide[kWidePrimes + 2]), total, out);
 }
 
 __global__ void k_wide_zero(radic_wide_result* out) {
@@ -344,16 +284,21 @@ int launch_wide_crt(const uint32_t* wide, radic_wide_result* out, unsigned long 
 }
 
 int launch_modp(const SinglePlan& p, const SingleArgs& a, cudaStream_t s) {
-  const void* k = pick(p, a.terms != nullptr);
+  const int use = a.terms ? kModpTerms : a.wide_out ? kModpWide : kModpDet;
+  const void* k = pick(p, use);
   if (!k) return RADIC_EUNSUPPORTED;
-  if (!allow_smem(k, smem_modp(p))) return RADIC_EUNSUPPORTED;
+  const size_t smem = smem_modp(p, use);
+  if (!allow_smem(k, smem)) return RADIC_EUNSUPPORTED;
   SingleArgs args = a;
-  PrefixTable tab = p.ptab;
+  const bool subtree = p.mapping == RADIC_MAP_PREFIX && use != kModpTerms;
+  PrefixTable tab = subtree ? p.stab[use] : p.ptab;
   void* params[] = {&args, &tab};
+  // the subtree kernel takes one prime per grid row; rows past the primes the
+  // bound asks for return at once
+  const dim3 grid(subtree ? p.sub_blocks[use] : p.blocks, subtree ? (use == kModpWide ? kWidePrimes : kMaxPrimes) : 1);
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(p.events);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return RADIC_ECUDA;
-  if (cudaLaunchKernel(k, dim3(p.blocks), dim3(p.threads), params, smem_modp(p), s) != cudaSuccess)
-    return RADIC_ECUDA;
+  if (cudaLaunchKernel(k, grid, dim3(p.threads), params, smem, s) != cudaSuccess) return RADIC_ECUDA;
   if (ev && cudaEventRecord(ev[1], s) != cudaSuccess) return RADIC_ECUDA;
   return RADIC_OK;
 }

@@ -12,24 +12,67 @@ namespace {
 
 constexpr int kMaxThreadsModp = 128;
 
-__constant__ uint32_t c_prime_table[kWidePrimes] = {
-    kPrimeTable[0],  kPrimeTable[1],  kPrimeTable[2],  kPrimeTable[3],  kPrimeTable[4],  kPrimeTable[5],
-    kPrimeTable[6],  kPrimeTable[7],  kPrimeTable[8],  kPrimeTable[9],  kPrimeTable[10], kPrimeTable[11],
-    kPrimeTable[12], kPrimeTable[13], kPrimeTable[14], kPrimeTable[15], kPrimeTable[16], kPrimeTable[17],
-    kPrimeTable[18], kPrimeTable[19], kPrimeTable[20], kPrimeTable[21], kPrimeTable[22], kPrimeTable[23],
-    kPrimeTable[24], kPrimeTable[25], kPrimeTable[26], kPrimeTable[27], kPrimeTable[28], kPrimeTable[29],
-    kPrimeTable[30], kPrimeTable[31]};
+// Constants of the primes, formed at compile time: the Montgomery constants
+// (inverse of p modulo 2^32, R and R^2 modulo p, R = 2^32), and for Garner's
+// mixed-radix form the partial products P_l = p_0 ... p_{l-1}: P_l and 1 / P_i
+// modulo p_i (times R, so that one Montgomery product applies them), and P_l
+// in base-2^32 limbs.
+struct PrimeConst {
+  uint32_t p, ninv, pinv, one, r2;  // ninv = -1/p, pinv = 1/p modulo 2^32
+};
+struct PrimeTables {
+  PrimeConst c[kWidePrimes];
+  uint32_t prod_mod[kWidePrimes][kWidePrimes];           // [l][i]: P_l R mod p_i
+  uint32_t prod_inv[kWidePrimes];                        // R / P_i mod p_i
+  uint32_t limbs[kWidePrimes + 1][RADIC_WIDE_LIMBS + 1];  // [l]: P_l
+};
 
-__host__ __device__ __forceinline__ uint32_t prime_at(int k) {
-#ifdef __CUDA_ARCH__
-  return c_prime_table[k];
-#else
-  return kPrimeTable[k];
-#endif
+constexpr PrimeTables make_prime_tables() {
+  PrimeTables t{};
+  for (int i = 0; i < kWidePrimes; ++i) {
+    const uint64_t p = kPrimeTable[i];
+    uint32_t x = static_cast<uint32_t>(p);  // Newton iteration x <- x (2 - p x) for 1/p modulo 2^32
+    for (int k = 0; k < 5; ++k) x *= 2u - static_cast<uint32_t>(p) * x;
+    const uint64_t r1 = (1ull << 32) % p;
+    t.c[i].p = static_cast<uint32_t>(p);
+    t.c[i].pinv = x;
+    t.c[i].ninv = 0u - x;
+    t.c[i].one = static_cast<uint32_t>(r1);
+    t.c[i].r2 = static_cast<uint32_t>(r1 * r1 % p);
+    uint64_t prod = 1;
+    for (int l = 0; l < kWidePrimes; ++l) {
+      t.prod_mod[l][i] = static_cast<uint32_t>(prod * r1 % p);
+      if (l == i) {  // prod = P_i: its inverse is P_i^(p-2)
+        uint64_t r = 1, b = prod, e = p - 2;
+        while (e) {
+          if (e & 1) r = r * b % p;
+          b = b * b % p;
+          e >>= 1;
+        }
+        t.prod_inv[i] = static_cast<uint32_t>(r * r1 % p);
+      }
+      prod = prod * (kPrimeTable[l] % p) % p;
+    }
+  }
+  t.limbs[0][0] = 1u;
+  for (int l = 0; l < kWidePrimes; ++l) {
+    uint64_t carry = 0;
+    for (int j = 0; j <= RADIC_WIDE_LIMBS; ++j) {
+      const uint64_t v = static_cast<uint64_t>(t.limbs[l][j]) * kPrimeTable[l] + carry;
+      t.limbs[l + 1][j] = static_cast<uint32_t>(v);
+      carry = v >> 32;
+    }
+  }
+  return t;
 }
 
+// read-only global memory: lanes read different entries
+static __device__ const PrimeTables c_primes = make_prime_tables();
+
+__device__ __forceinline__ uint32_t prime_at(int k) { return __ldg(&c_primes.c[k].p); }
+
 struct Mont {
-  uint32_t p, pinv, one, r2;
+  uint32_t p, pinv, one, r2;  // pinv = -1/p modulo 2^32
   uint64_t p2;
 };
 
@@ -53,16 +96,14 @@ __device__ __forceinline__ uint32_t add_mod(uint32_t a, uint32_t b, uint32_t p) 
 }
 __device__ __forceinline__ uint32_t neg_mod(uint32_t a, uint32_t p) { return a ? p - a : 0u; }
 
-__device__ inline Mont make_mont(uint32_t p) {
+__device__ __forceinline__ Mont make_mont(int k) {
+  const PrimeConst c = c_primes.c[k];
   Mont mp;
-  mp.p = p;
-  uint32_t x = p;  // inverse of p modulo 2^32 by Newton iteration x <- x (2 - p x)
-  for (int i = 0; i < 5; ++i) x *= 2u - p * x;
-  mp.pinv = 0u - x;
-  const uint64_t r1 = (1ull << 32) % p;
-  mp.one = static_cast<uint32_t>(r1);
-  mp.r2 = static_cast<uint32_t>((r1 * r1) % p);
-  mp.p2 = static_cast<uint64_t>(p) * p;
+  mp.p = c.p;
+  mp.pinv = c.ninv;
+  mp.one = c.one;
+  mp.r2 = c.r2;
+  mp.p2 = static_cast<uint64_t>(c.p) * c.p;
   return mp;
 }
 
@@ -76,7 +117,27 @@ __device__ inline uint32_t mpow(uint32_t x, uint32_t e, const Mont& mp) {
   }
   return r;
 }
-__device__ inline uint32_t minv(uint32_t x, const Mont& mp) { return mpow(x, mp.p - 2u, mp); }
+// x^(p-2) = 1/x (0 for 0) in Montgomery form.  p = 2^31 - d with d < 2^10, so
+// the exponent 2^31 - (d + 2) is 21 ones followed by ten bits: the ones by
+// doubling (x^(2^k - 1) for k = 1, 2, 4, 5, 10, 20, 21), the bits one at a
+// time; about 42 dependent products instead of 60.
+static_assert(kPrimeTable[kWidePrimes - 1] > (1u << 31) - (1u << 10) + 2u, "leading ones of p - 2");
+__device__ inline uint32_t minv(uint32_t x, const Mont& mp) {
+  auto sq = [&](uint32_t a, int k) {
+    for (int i = 0; i < k; ++i) a = mmul(a, a, mp);
+    return a;
+  };
+  const uint32_t a2 = mmul(sq(x, 1), x, mp), a4 = mmul(sq(a2, 2), a2, mp), a5 = mmul(sq(a4, 1), x, mp);
+  const uint32_t a10 = mmul(sq(a5, 5), a5, mp), a20 = mmul(sq(a10, 10), a10, mp);
+  uint32_t r = mmul(sq(a20, 1), x, mp);
+  const uint32_t e = mp.p - 2u;
+#pragma unroll 1
+  for (int b = 9; b >= 0; --b) {
+    r = mmul(r, r, mp);
+    if ((e >> b) & 1u) r = mmul(r, x, mp);
+  }
+  return r;
+}
 
 __device__ inline uint64_t mix64(uint64_t z) {  // SplitMix64 finaliser
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
@@ -85,34 +146,48 @@ __device__ inline uint64_t mix64(uint64_t z) {  // SplitMix64 finaliser
 }
 
 // Shared-memory layout: binom | K x (n x cs) residues (column-major, Montgomery
-// form) | m x n scratch rows | scratch words for reductions.
+// form) | 2 x (m x n) scratch rows | m x m triangular factors | row bounds |
+// scratch words for reductions | counts | Montgomery constants | row exponents.
 __host__ __device__ inline size_t modp_smem_bytes(int n, int m, int cs, int threads) {
   size_t off = ((size_t)(n + 1) * (m + 1) * 8 + 15) / 16 * 16;
   off += (size_t)kMaxPrimes * n * cs * 4;
-  off += ((size_t)m * n * 4 + 15) / 16 * 16;
+  off += (2 * (size_t)m * n * 4 + 15) / 16 * 16;
+  off += ((size_t)m * m * 4 + 15) / 16 * 16;
+  off += (size_t)(m + 1) * 12;
   off += (size_t)(threads / 32) * kMaxPrimes * 4;
+  off = (off + 15) / 16 * 16;
   off += 64 + kMaxPrimes * sizeof(Mont);
-  off += (size_t)kMaxM * 4;  // row exponents of floating-point inputs
-  return off;
+  off += (size_t)kMaxM * 8;  // row exponents and widths of floating-point inputs
+  return (off + 15) / 16 * 16;
 }
 
 struct ModpSmem {
   uint64_t* binom;
   uint32_t* As;  // prime k at As + k * n * cs
   uint32_t* rows;
+  uint32_t* tri;
+  double* row_bits;
+  float* bits32;
   uint32_t* scratch;
   int* misc;  // [0] primes the bound needs, [1] total row exponent, [2] non-finite flag
   Mont* mont;
-  int* row_e;  // floating-point inputs: row i times 2^-row_e[i] is integer
+  int* row_e;  // floating-point inputs: row i times 2^-row_e[i] is integer, of width row_e[m + i]
   __device__ ModpSmem(unsigned char* base, int n, int m, int cs, int threads) {
     size_t off = ((size_t)(n + 1) * (m + 1) * 8 + 15) / 16 * 16;
     binom = reinterpret_cast<uint64_t*>(base);
     As = reinterpret_cast<uint32_t*>(base + off);
     off += (size_t)kMaxPrimes * n * cs * 4;
     rows = reinterpret_cast<uint32_t*>(base + off);
-    off += ((size_t)m * n * 4 + 15) / 16 * 16;
+    off += (2 * (size_t)m * n * 4 + 15) / 16 * 16;
+    tri = reinterpret_cast<uint32_t*>(base + off);
+    off += ((size_t)m * m * 4 + 15) / 16 * 16;
+    row_bits = reinterpret_cast<double*>(base + off);
+    off += (size_t)(m + 1) * 8;
+    bits32 = reinterpret_cast<float*>(base + off);
+    off += (size_t)(m + 1) * 4;
     scratch = reinterpret_cast<uint32_t*>(base + off);
     off += (size_t)(threads / 32) * kMaxPrimes * 4;
+    off = (off + 15) / 16 * 16;
     misc = reinterpret_cast<int*>(base + off);
     off += 64;
     mont = reinterpret_cast<Mont*>(base + off);
@@ -155,38 +230,43 @@ __device__ __forceinline__ double load_fp(const void* A, int dtype, long long id
 }
 __device__ __forceinline__ bool is_fp_dtype(int dtype) { return dtype == kF32 || dtype == kF64; }
 
-// 2^k mod p, k >= 0 (square and multiply).
-__device__ inline uint64_t pow2_mod(int k, uint64_t p) {
-  uint64_t r = 1, b = 2 % p;
-  while (k) {
-    if (k & 1) r = r * b % p;
-    b = b * b % p;
-    k >>= 1;
-  }
-  return r % p;
+// Montgomery form of a 64-bit integer: hi 2^32 + lo, 2^32 = R.
+__device__ __forceinline__ uint32_t to_mont64(uint64_t x, const Mont& mp) {
+  const uint32_t hi = mmul(static_cast<uint32_t>(x >> 32), mp.r2, mp), lo = mmul(static_cast<uint32_t>(x), mp.r2, mp);
+  return add_mod(mmul(hi, mp.r2, mp), lo, mp.p);
 }
 
-// Residue of the integer x * 2^-e modulo p (e at most the exponent of x's
-// lowest set bit, so that the shift below drops only zeros).
-__device__ inline uint32_t fp_residue(double x, int e, uint32_t p) {
+// Residue (normal form) of the integer x * 2^-e modulo p (e at most the
+// exponent of x's lowest set bit, so that the shift below drops only zeros).
+__device__ inline uint32_t fp_residue(double x, int e, const Mont& mp) {
   const FpBits f = fp_bits(x);
   if (f.mant == 0) return 0u;
-  uint64_t r;
+  uint32_t r;
   if (f.t >= e) {
-    r = (f.mant % p) * pow2_mod(f.t - e, p) % p;
+    const uint32_t two = add_mod(mp.one, mp.one, mp.p);
+    r = mmul(to_mont64(f.mant, mp), mpow(two, static_cast<uint32_t>(f.t - e), mp), mp);
   } else {
-    r = (f.mant >> (e - f.t)) % p;
+    r = to_mont64(f.mant >> (e - f.t), mp);
   }
-  return (f.neg && r) ? static_cast<uint32_t>(p - r) : static_cast<uint32_t>(r);
+  r = redc(r, mp.p, mp.pinv);
+  return f.neg ? neg_mod(r, mp.p) : r;
 }
 
-// Row exponents e_i (into row_e) and, per row, the bits of a bound on the
-// Euclidean norm of the integer row: |entry| < 2^(top_i + 1 - e_i) with top_i
-// the exponent of the highest set bit, so ||M_i|| < sqrt(n) 2^(top_i + 1 - e_i).
-// A zero row has e_i = 0 and no bits (all its minors are zero).  Sets
-// *nonfinite (shared) when an entry is infinite or NaN.
+// Residue (normal form) of a 32-bit integer.
+__device__ __forceinline__ uint32_t int_residue(long long v, uint32_t p) {
+  if (v < 0) v += p;
+  if (v < 0) v += p;  // -2^31 needs p twice for the primes below 2^31
+  return static_cast<uint32_t>(v >= (long long)p ? v - p : v);
+}
+
+// Row exponents e_i (row_e[i]) and, per row, the width w_i (row_e[m + i]) of
+// a bound on the Euclidean norm of the integer row: |entry| < 2^w_i with
+// w_i = top_i + 1 - e_i, top_i the exponent of the highest set bit, so
+// ||M_i|| < sqrt(n) 2^w_i.  A zero row has e_i = 0 and width 0, for no bits
+// (all its minors are zero).  Sets *nonfinite (shared) when an entry is
+// infinite or NaN.
 __device__ inline void fp_row_scales(const void* A, int dtype, int m, int n, long long lda, int* row_e,
-                                     double* row_bits, int* nonfinite) {
+                                     int* nonfinite) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int i = warp; i < m; i += nw) {
     int lo = 0x7fffffff, hi = -0x7fffffff;
@@ -206,33 +286,129 @@ __device__ inline void fp_row_scales(const void* A, int dtype, int m, int n, lon
     if (lane == 0) {
       const bool zero = hi == -0x7fffffff;
       row_e[i] = zero ? 0 : lo;
-      row_bits[i] = zero ? 0.0 : static_cast<double>(hi + 1 - lo) + 0.5 * log2(static_cast<double>(n));
+      row_e[m + i] = zero ? 0 : hi + 1 - lo;
       if (bad) *nonfinite = 1;
     }
   }
 }
 
-// Number of primes for |det_R(A)| <= C(n,m) prod_i ||row_i||_2 (Hadamard's
-// inequality for every minor), plus a sign bit and a margin.  One warp per
-// row computes the squared row norms into row_sq[]; thread 0 sums the logs.
-__device__ inline int primes_needed(const void* A, int dtype, int m, int n, long long lda, double log2_count,
-                                    double* row_sq) {
+// Bits of a bound on |det_R(A)| from the rows: C(n,m) prod_i ||row_i||_2
+// (Hadamard's inequality for every minor).  Integer rows by their norms, one
+// warp per row; floating-point rows by the widths of fp_row_scales.  Type F:
+// double as the count of primes is defined, float for the estimate below.
+// bits: m + 1 words of shared scratch, left with the rows' bits and
+// log2 C(n,m); ends with a barrier.
+template <typename F>
+__device__ inline void hadamard_bits(const SingleArgs& a, int m, double count, const int* row_e, F* bits) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = warp; i < m; i += nw) {
-    double s = 0.0;
-    for (int j = lane; j < n; j += 32) {
-      const double v = static_cast<double>(load_int(A, dtype, (long long)i * lda + j));
-      s += v * v;
+  if (is_fp_dtype(a.dtype)) {
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+      const int w = row_e[m + i];
+      bits[i] = w == 0 ? F(0) : static_cast<F>(w) + F(0.5) * log2(static_cast<F>(a.n));
     }
+  } else {
+    for (int i = warp; i < m; i += nw) {
+      F s = F(0);
+      for (int j = lane; j < a.n; j += 32) {
+        const F v = static_cast<F>(load_int(a.A, a.dtype, (long long)i * a.lda + j));
+        s += v * v;
+      }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
-    if (lane == 0) row_sq[i] = s;
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+      if (lane == 0) bits[i] = F(0.5) * log2(max(s, F(1)));
+    }
+  }
+  if (threadIdx.x == 0) bits[m] = log2(max(static_cast<F>(count), F(1)));
+  __syncthreads();
+}
+
+// Number of primes for that bound, plus a sign bit and a margin, into
+// *needed, and the total row exponent of floating-point inputs into *esum;
+// row_e holds the row exponents and widths (2 m words).  The count is defined in binary64, whose
+// logarithms and sums are long chains on a slow pipe (the larger part of a
+// small call: 3 x 12 took 16.4 us a call with them).  The block therefore
+// sums the bits in binary32 first, whose error is below kNear of a prime
+// (at most 33 sums of at most 1100 bits for up to 32 primes: 2e-3 bits, 7e-5
+// primes, plus the norms' 1e-5), and redoes it in binary64 only when a count
+// boundary is that close.  row_bits: m + 1 words of shared scratch, bits32:
+// m + 1.  Ends with a barrier.
+__device__ inline void scale_and_count_primes(const SingleArgs& a, int m, double count, double* row_bits,
+                                              float* bits32, int* row_e, int* nonfinite, int* needed, int* esum) {
+  constexpr float kNear = 1e-3f;
+  const bool fp = is_fp_dtype(a.dtype);
+  if (fp) {
+    if (threadIdx.x == 0) *nonfinite = 0;
+    __syncthreads();
+    fp_row_scales(a.A, a.dtype, m, a.n, a.lda, row_e, nonfinite);
+    __syncthreads();
+  }
+  hadamard_bits<float>(a, m, count, row_e, bits32);
+  float est = 0.0f;
+  int es = 0;
+  for (int i = 0; i <= m; ++i) est += bits32[i];
+  if (fp)
+    for (int i = 0; i < m; ++i) es += row_e[i];
+  const float q = (est + 2.0f) * (1.0f / 30.99f);
+  int k = static_cast<int>(ceilf(q));
+  if (fabsf(q - rintf(q)) <= kNear || !(q < 1e6f)) {  // the same in every thread
+    hadamard_bits<double>(a, m, count, row_e, row_bits);
+    double bits = row_bits[m];
+    for (int i = 0; i < m; ++i) bits += row_bits[i];
+    k = static_cast<int>(ceil((bits + 2.0) / 30.99));
+  }
+  if (threadIdx.x == 0) {
+    *needed = k < 1 ? 1 : k;
+    *esum = es;
+    if (fp && *nonfinite) atomicExch(&a.hdr->status, RADIC_EINVAL);  // an entry is not finite
   }
   __syncthreads();
-  double bits = log2_count;
-  for (int i = 0; i < m; ++i) bits += 0.5 * log2(fmax(row_sq[i], 1.0));
-  const int k = static_cast<int>(ceil((bits + 2.0) / 30.99));
-  return k < 1 ? 1 : k;
+}
+
+// (T A mod p) in Montgomery form into As (column-major, column stride cs,
+// padding rows zero) for the prime mp: T = L U with L unit lower and U unit
+// upper triangular, entries from a hash of (slot, row, column).  Rows of U A
+// and of L (U A) are independent sums, so each product is one pass of the
+// block over the m n entries.  With alt_sign, odd columns are negated (the
+// column parities of Eq. (1)).  tri: m x m words, rows: 2 m n words of shared
+// scratch; row_e as from scale_and_count_primes.
+__device__ inline void stage_prime(const SingleArgs& a, int m, int cs, int slot, const Mont& mp, const int* row_e,
+                                   uint32_t* tri, uint32_t* rows, uint32_t* As, bool alt_sign) {
+  const int n = a.n, mn = m * n;
+  const bool fp = is_fp_dtype(a.dtype);
+  uint32_t* ua = rows + mn;
+  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
+    const int i = idx / m, l = idx - i * m;
+    const uint64_t h = l > i ? mix64(0x9e3779b97f4a7c15ull * (uint64_t)(slot * 4096 + i * 64 + l) + 1ull)
+                             : mix64(0xd1b54a32d192ed03ull * (uint64_t)(slot * 4096 + i * 64 + l) + 7ull);
+    const uint32_t r = static_cast<uint32_t>(h >> 33);  // 31 bits
+    tri[idx] = r >= mp.p ? r - mp.p : r;
+  }
+  for (int idx = threadIdx.x; idx < mn; idx += blockDim.x) {
+    const int i = idx / n, j = idx - i * n;
+    const long long at = (long long)i * a.lda + j;
+    rows[idx] = fp ? fp_residue(load_fp(a.A, a.dtype, at), row_e[i], mp)
+                   : int_residue(load_int(a.A, a.dtype, at), mp.p);
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < mn; idx += blockDim.x) {
+    const int i = idx / n, j = idx - i * n;
+    uint32_t acc = rows[idx];
+    for (int l = i + 1; l < m; ++l) acc = add_mod(acc, mmul(tri[i * m + l], rows[l * n + j], mp), mp.p);
+    ua[idx] = acc;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * cs; idx += blockDim.x) {
+    const int j = idx / cs, i = idx - j * cs;
+    uint32_t v = 0u;
+    if (i < m) {
+      v = ua[i * n + j];
+      for (int l = 0; l < i; ++l) v = add_mod(v, mmul(tri[i * m + l], ua[l * n + j], mp), mp.p);
+      v = mmul(v, mp.r2, mp);
+      if (alt_sign && (j & 1)) v = neg_mod(v, mp.p);
+    }
+    As[idx] = v;
+  }
+  __syncthreads();
 }
 
 // Stage binom and, for each prime of the pass, (T A mod p) in Montgomery
@@ -244,85 +420,13 @@ __device__ inline int stage_modp(const SingleArgs& a, const ModpSmem& sm, int m,
   const int base = a.prime_base;
   build_binom(sm.binom, n, m);
   if (threadIdx.x < kMaxPrimes && base + (int)threadIdx.x < kWidePrimes)
-    sm.mont[threadIdx.x] = make_mont(prime_at(base + threadIdx.x));
-  const bool fp = is_fp_dtype(a.dtype);
-  {
-    // the rows scratch (m x n words) is free until the residues are staged
-    double* row_sq = reinterpret_cast<double*>(sm.rows);
-    const double cnt = static_cast<double>(sm.binom[n * (m + 1) + m]);
-    if (fp) {
-      if (threadIdx.x == 0) sm.misc[2] = 0;
-      __syncthreads();
-      fp_row_scales(a.A, a.dtype, m, n, a.lda, sm.row_e, row_sq, &sm.misc[2]);
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double bits = log2(fmax(cnt, 1.0));
-        int esum = 0;
-        for (int i = 0; i < m; ++i) {
-          bits += row_sq[i];
-          esum += sm.row_e[i];
-        }
-        const int k = static_cast<int>(ceil((bits + 2.0) / 30.99));
-        sm.misc[0] = k < 1 ? 1 : k;
-        sm.misc[1] = esum;
-        if (sm.misc[2]) atomicExch(&a.hdr->status, RADIC_EINVAL);  // an entry is not finite
-      }
-    } else {
-      const int need = primes_needed(a.A, a.dtype, m, n, a.lda, log2(fmax(cnt, 1.0)), row_sq);
-      if (threadIdx.x == 0) {
-        sm.misc[0] = need;
-        sm.misc[1] = 0;
-      }
-    }
-  }
-  __syncthreads();
+    sm.mont[threadIdx.x] = make_mont(base + threadIdx.x);
+  scale_and_count_primes(a, m, static_cast<double>(sm.binom[n * (m + 1) + m]), sm.row_bits, sm.bits32, sm.row_e,
+                         &sm.misc[2], &sm.misc[0], &sm.misc[1]);
   *needed = sm.misc[0];
   const int K = max(0, min(min(sm.misc[0], kWidePrimes) - base, kMaxPrimes));
-  for (int k = 0; k < K; ++k) {
-    const uint32_t p = prime_at(base + k);
-    for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) {
-      const int i = idx / n, j = idx - i * n;
-      if (fp) {
-        sm.rows[idx] = fp_residue(load_fp(a.A, a.dtype, (long long)i * a.lda + j), sm.row_e[i], p);
-      } else {
-        long long v = load_int(a.A, a.dtype, (long long)i * a.lda + j) % (long long)p;
-        if (v < 0) v += p;
-        sm.rows[idx] = static_cast<uint32_t>(v);
-      }
-    }
-    __syncthreads();
-    // rows <- U rows (unit upper: row i += sum_{l > i} U_il row_l), ascending i
-    for (int i = 0; i < m; ++i) {
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        uint64_t acc = sm.rows[i * n + j];
-        for (int l = i + 1; l < m; ++l) {
-          const uint64_t u = mix64(0x9e3779b97f4a7c15ull * (uint64_t)(k * 4096 + i * 64 + l) + 1ull) % p;
-          acc = (acc + u * sm.rows[l * n + j]) % p;
-        }
-        sm.rows[i * n + j] = static_cast<uint32_t>(acc);
-      }
-      __syncthreads();
-    }
-    // rows <- L rows (unit lower: row i += sum_{l < i} L_il row_l), descending i
-    for (int i = m - 1; i >= 0; --i) {
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        uint64_t acc = sm.rows[i * n + j];
-        for (int l = 0; l < i; ++l) {
-          const uint64_t u = mix64(0xd1b54a32d192ed03ull * (uint64_t)(k * 4096 + i * 64 + l) + 7ull) % p;
-          acc = (acc + u * sm.rows[l * n + j]) % p;
-        }
-        sm.rows[i * n + j] = static_cast<uint32_t>(acc);
-      }
-      __syncthreads();
-    }
-    const Mont mp = make_mont(p);
-    uint32_t* dst = sm.As + (size_t)k * n * cs;
-    for (int idx = threadIdx.x; idx < n * cs; idx += blockDim.x) {
-      const int j = idx / cs, i = idx - j * cs;
-      dst[idx] = (i < m) ? mmul(sm.rows[i * n + j], mp.r2, mp) : 0u;
-    }
-    __syncthreads();
-  }
+  for (int k = 0; k < K; ++k)
+    stage_prime(a, m, cs, k, sm.mont[k], sm.row_e, sm.tri, sm.rows, sm.As + (size_t)k * n * cs, false);
   return K;
 }
 
@@ -423,36 +527,25 @@ __device__ inline void block_reduce_modp(uint32_t (&r)[kMaxPrimes], int K, uint3
   }
 }
 
-__device__ inline uint64_t powmod64(uint64_t b, uint64_t e, uint64_t p) {
-  uint64_t r = 1 % p;
-  b %= p;
-  while (e) {
-    if (e & 1) r = (r * b) % p;
-    b = (b * b) % p;
-    e >>= 1;
-  }
-  return r;
-}
-
 // Garner reconstruction of the signed value in (-P/2, P/2].
 __device__ inline void crt_write(radic_result* out, const uint32_t* res, int K, int needed, int status,
                                  unsigned long long total, int escale) {
-  uint64_t v[kMaxPrimes];
-  for (int i = 0; i < K; ++i) {
-    const uint64_t p = prime_at(i);
-    // value of the digits so far modulo p, and prod_{l<i} p_l modulo p
-    uint64_t acc = 0, prod = 1;
-    for (int l = 0; l < i; ++l) {
-      acc = (acc + v[l] * prod) % p;
-      prod = (prod * (prime_at(l) % p)) % p;
-    }
-    const uint64_t diff = (res[i] + p - acc) % p;
-    v[i] = (diff * powmod64(prod, p - 2, p)) % p;
+  uint32_t v[kMaxPrimes];
+#pragma unroll
+  for (int i = 0; i < kMaxPrimes; ++i) {
+    const Mont mp = make_mont(i);
+    uint32_t acc = 0u;  // value of the digits so far modulo p
+#pragma unroll
+    for (int l = 0; l < i; ++l) acc = add_mod(acc, mmul(v[l], c_primes.prod_mod[l][i], mp), mp.p);
+    v[i] = mmul(add_mod(res[i], neg_mod(acc, mp.p), mp.p), c_primes.prod_inv[i], mp);
   }
   unsigned __int128 x = 0, big = 1;
-  for (int i = 0; i < K; ++i) {
-    x += static_cast<unsigned __int128>(v[i]) * big;
-    big *= prime_at(i);
+#pragma unroll
+  for (int i = 0; i < kMaxPrimes; ++i) {
+    if (i < K) {
+      x += static_cast<unsigned __int128>(v[i]) * big;
+      big *= prime_at(i);
+    }
   }
   __int128 sx = static_cast<__int128>(x);
   if (x > big / 2) sx = static_cast<__int128>(x) - static_cast<__int128>(big);
@@ -473,6 +566,96 @@ __device__ inline void crt_write(radic_result* out, const uint32_t* res, int K, 
   out->tier = kModeExact;
   out->exact_exp = escale;
   for (int i = 0; i < 5; ++i) out->reserved[i] = 0;
+}
+
+// Wide exact result from the residues modulo the first K primes (lane i
+// holds residue i; K <= 32), by one whole warp.  Mixed-radix digits v_l
+// (Garner): step l fixes v_l in lane l, and the later lanes add v_l P_l to
+// their value modulo their own prime.  The integer is sum_l v_l P_l: lane j
+// adds limb j of every term (the P_l are compile-time constants), then the
+// warp resolves the carries.  The symmetric range (-M/2, M/2), M the product
+// of the primes, gives the sign.  (Written serially, with an exponentiation
+// per digit and a limb-by-limb Horner rule, this took 245 us for 15 primes;
+// by a warp but with 64-bit divisions still 44 us.)
+static_assert(RADIC_WIDE_LIMBS == 32 && kWidePrimes == 32, "one lane per limb and prime; kAhead divides it");
+
+// x + carry-in from the lane below until no lane carries; lane 31's carry is lost.
+__device__ inline uint32_t warp_resolve_carry(uint64_t x, int lane) {
+  for (;;) {
+    const uint32_t c = static_cast<uint32_t>(x >> 32);
+    if (!__any_sync(kFull, c != 0u)) return static_cast<uint32_t>(x);
+    const uint32_t in = __shfl_up_sync(kFull, c, 1);
+    x = (x & 0xffffffffull) + (lane > 0 ? in : 0u);
+  }
+}
+// Limbs of a - b (a >= b), lane j holding limb j.
+__device__ inline uint32_t warp_limbs_sub(uint32_t a, uint32_t b, int lane) {
+  long long t = static_cast<long long>(a) - b;
+  for (;;) {
+    const int borrow = t < 0;
+    if (!__any_sync(kFull, borrow)) return static_cast<uint32_t>(t);
+    if (borrow) t += 1ll << 32;
+    const int in = __shfl_up_sync(kFull, borrow, 1);
+    if (lane > 0) t -= in;
+  }
+}
+
+__device__ inline void wide_crt_warp(uint32_t res, int K, int needed, int escale, int status, unsigned long long total,
+                                     radic_wide_result* out) {
+  const int lane = threadIdx.x & 31;
+  const Mont mp = make_mont(lane);
+  const uint32_t inv = c_primes.prod_inv[lane];
+  uint32_t acc = 0u;
+  uint64_t lo = 0;   // limb j of the sum, 96 bits
+  uint32_t hi = 0u;
+  // constants are fetched kAhead steps at a time, ahead of the digit chain
+  constexpr int kAhead = 8;
+  for (int l0 = 0; l0 < K; l0 += kAhead) {
+    uint32_t pm[kAhead], lm[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      pm[u] = __ldg(&c_primes.prod_mod[l0 + u][lane]);
+      lm[u] = __ldg(&c_primes.limbs[l0 + u][lane]);
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      if (l0 + u < K) {
+        const uint32_t d = mmul(add_mod(res, neg_mod(acc, mp.p), mp.p), inv, mp);
+        const uint32_t v = __shfl_sync(kFull, d, l0 + u);
+        if (lane > l0 + u) acc = add_mod(acc, mmul(v, pm[u], mp), mp.p);
+        const uint64_t t = static_cast<uint64_t>(v) * lm[u];
+        lo += t;
+        hi += lo < t ? 1u : 0u;
+      }
+    }
+  }
+  // x = sum over lanes of (hi 2^64 + lo) 2^(32 lane)
+  const uint32_t mid = __shfl_up_sync(kFull, static_cast<uint32_t>(lo >> 32), 1);
+  const uint32_t top = __shfl_up_sync(kFull, hi, 2);
+  const uint32_t x = warp_resolve_carry((lo & 0xffffffffull) + (lane > 0 ? mid : 0u) + (lane > 1 ? top : 0u), lane);
+  // d = M - x; the value is x when x < d (that is x < M/2), else -(M - x).
+  // M < 2^(31 * 32) fits the 32 limbs.
+  const uint32_t d = warp_limbs_sub(c_primes.limbs[K][lane], x, lane);
+  const unsigned lt = __ballot_sync(kFull, x < d), gt = __ballot_sync(kFull, x > d);
+  const bool x_less = lt > gt;  // the highest limb that differs decides
+  const uint32_t mag = x_less ? x : d;
+  const unsigned used = __ballot_sync(kFull, mag != 0u);
+  const int nl = 32 - __clz(static_cast<int>(used));
+  out->limbs[lane] = mag;
+  double val = 0.0;
+  const int low = nl > 3 ? nl - 3 : 0;
+  for (int i = nl - 1; i >= low; --i) val = val * 4294967296.0 + static_cast<double>(__shfl_sync(kFull, mag, i));
+  if (lane == 0) {
+    const int sgn = nl == 0 ? 0 : (x_less ? 1 : -1);
+    out->value = sgn < 0 ? -ldexp(val, 32 * low + escale) : ldexp(val, 32 * low + escale);
+    out->status = (needed > kWidePrimes) ? RADIC_EOVERFLOW : status;
+    out->n_primes = K;
+    out->exact_exp = escale;
+    out->sign = sgn;
+    out->n_limbs = nl;
+    out->minors = static_cast<long long>(total);
+    out->reserved = 0;
+  }
 }
 
 // Last-block epilogue shared by both mappings.

@@ -1,5 +1,7 @@
-// Exact path, prefix mapping: the minors of one (m-D)-column prefix share
-// its non-dividing elimination mod p (see the comment of k_modp_prefix).
+// Exact path, prefix mapping, per-minor terms (radic_terms): the minors of one
+// (m-D)-column prefix share its non-dividing elimination mod p (see the
+// comment of k_modp_prefix).  The determinant itself sums whole subtrees
+// (radic_modp_subtree.cuh).
 #include "radic_modp.cuh"
 
 namespace radic {
@@ -18,9 +20,9 @@ namespace {
 // complement of x and s = prod_k pi_k.  The true pivots t_k satisfy
 // pi_k = t_k prod_{j<k} pi_j, so every leaf minor of the prefix is
 //   det = +- prod_k t_k det(Z) = +- det(s Z) / (s^(D-1) prod_k prod_{j<k} pi_j),
-// one denominator for the whole subtree: each lane keeps its sum as one
-// fraction and inverts once at the end.  A prefix singular mod p has a zero
-// pivot after the search, s = 0, and all its minors are 0 mod p.
+// one denominator for the whole subtree, inverted once per prefix and prime.
+// A prefix singular mod p has a zero pivot after the search, s = 0, and all
+// its minors are 0 mod p.
 // ---------------------------------------------------------------------------
 template <int M, int D, int CS>
 __device__ __forceinline__ void modp_prefix_factor(const uint32_t* __restrict__ As, const int (&c)[M - D],
@@ -111,40 +113,35 @@ __device__ __forceinline__ uint32_t modp_dot(const uint32_t (&y)[3], const uint3
   return add_mod(redc(t, mp.p, mp.pinv), mmul(y[2], w[2], mp), mp.p);
 }
 
-// Sum (Montgomery form) of a lane's share of the leaves of one prefix, one
-// candidate column at a time; lane `sub` of `lp` takes the leaves whose
-// second-to-last column index is congruent to sub.  Leaf values are added as
-// integers and reduced once per column (fewer than 2^31 addends of < p).
-// With a terms sink, each leaf's signed term (times inv_den) is stored.
-template <int M, int D, bool kTerms>
-__device__ __forceinline__ uint32_t modp_prefix_leaves(const uint32_t* __restrict__ As, int cs, const uint64_t* binom,
-                                                       int n, int v, const uint32_t (&a)[M][M - D],
-                                                       const int (&idx)[M], const uint32_t (&piv)[M - D],
-                                                       const Mont& mp, const ZBuf<uint32_t, D>& zb, int sub, int lp,
-                                                       bool negp, uint32_t inv_den,
-                                                       unsigned long long rank_prefix, const TermsSink& ts,
-                                                       uint32_t* terms, bool act) {
+// Signed terms (times inv_den) of a lane's share of the leaves of one prefix,
+// one candidate column at a time; lane `sub` of `lp` takes the leaves whose
+// second-to-last column index is congruent to sub.  Terms outside the
+// requested window of ranks are dropped.
+template <int M, int D>
+__device__ __forceinline__ void modp_prefix_leaves(const uint32_t* __restrict__ As, int cs, const uint64_t* binom,
+                                                   int n, int v, const uint32_t (&a)[M][M - D],
+                                                   const int (&idx)[M], const uint32_t (&piv)[M - D],
+                                                   const Mont& mp, const ZBuf<uint32_t, D>& zb, int sub, int lp,
+                                                   bool negp, uint32_t inv_den, unsigned long long rank_prefix,
+                                                   const TermsSink& ts, uint32_t* terms, bool act) {
   const int k = n - 1 - v, bs = M + 1;
-  uint32_t S = 0u;
+  auto emit = [&](uint32_t d, unsigned long long rank) {
+    const unsigned long long rk = ts.qtot - 1 - rank;
+    if (act && rk >= ts.q0 && rk < ts.q0 + ts.count) {
+      const uint32_t t = redc(mmul(d, inv_den, mp), mp.p, mp.pinv);
+      terms[rk - ts.q0] = negp ? neg_mod(t, mp.p) : t;
+    }
+  };
   for (int q = 0; q < k; ++q) {
     const int col = v + 1 + q;
     uint32_t z[D];
     modp_prefix_column<M, D>(As + col * cs, col, a, idx, piv, mp, z);
-    uint64_t csum = 0;
     const unsigned long long rk_col = rank_prefix + rank_part(binom, bs, n, col, 1);
     if constexpr (D == 2) {
       for (int q2 = sub; q2 < q; q2 += lp) {
         uint32_t y[2];
         zb.get(q2, y);
-        const uint32_t d = modp_det2(y, z, mp);
-        csum += d;
-        if constexpr (kTerms) {
-          const unsigned long long rk = ts.qtot - 1 - (rk_col + rank_part(binom, bs, n, v + 1 + q2, 2));
-          if (act && rk >= ts.q0 && rk < ts.q0 + ts.count) {
-            uint32_t t = redc(mmul(d, inv_den, mp), mp.p, mp.pinv);
-            terms[rk - ts.q0] = negp ? neg_mod(t, mp.p) : t;
-          }
-        }
+        emit(modp_det2(y, z, mp), rk_col + rank_part(binom, bs, n, v + 1 + q2, 2));
       }
     } else {
       for (int q2 = sub; q2 < q; q2 += lp) {
@@ -156,26 +153,15 @@ __device__ __forceinline__ uint32_t modp_prefix_leaves(const uint32_t* __restric
         for (int q1 = 0; q1 < q2; ++q1) {
           uint32_t y1[3];
           zb.get(q1, y1);
-          const uint32_t d = modp_dot(y1, w, mp);
-          csum += d;
-          if constexpr (kTerms) {
-            const unsigned long long rk = ts.qtot - 1 - (rk2 + rank_part(binom, bs, n, v + 1 + q1, 3));
-            if (act && rk >= ts.q0 && rk < ts.q0 + ts.count) {
-              uint32_t t = redc(mmul(d, inv_den, mp), mp.p, mp.pinv);
-              terms[rk - ts.q0] = negp ? neg_mod(t, mp.p) : t;
-            }
-          }
+          emit(modp_dot(y1, w, mp), rk2 + rank_part(binom, bs, n, v + 1 + q1, 3));
         }
       }
     }
     zb.put(q, z);
-    // sum of Montgomery-form values -> normal form (redc) -> Montgomery form
-    S = add_mod(S, mmul(redc(csum, mp.p, mp.pinv), mp.r2, mp), mp.p);
   }
-  return S;
 }
 
-template <int M, int D, bool kTerms>
+template <int M, int D>
 __global__ void __launch_bounds__(kMaxThreadsModp) k_modp_prefix(SingleArgs a, PrefixTable tab) {
   static_assert(M > D, "the prefix needs at least one column");
   constexpr int P = M - D;
@@ -186,20 +172,13 @@ __global__ void __launch_bounds__(kMaxThreadsModp) k_modp_prefix(SingleArgs a, P
   const ZBuf<uint32_t, D> zb(smem_raw + modp_smem_bytes(n, M, CS, blockDim.x), threadIdx.x, blockDim.x, n - M + D);
   int needed;
   const int K = stage_modp(a, sm, M, CS, &needed);
-  if (K == 0) return;  // a wide pass whose primes the bound does not need
 
   const int lane = threadIdx.x & 31;
   const unsigned long long gwarp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned long long nwarps = (unsigned long long)gridDim.x * blockDim.x / 32;
   const int bs = M + 1;
-  TermsSink ts{nullptr, a.q0, a.count, sm.binom[n * bs + M], 0};
+  const TermsSink ts{nullptr, a.q0, a.count, sm.binom[n * bs + M], 0};
 
-  uint32_t N[kMaxPrimes], Dn[kMaxPrimes];
-#pragma unroll
-  for (int k = 0; k < kMaxPrimes; ++k) {
-    N[k] = 0u;
-    Dn[k] = sm.mont[k].one;
-  }
   for (unsigned long long t = gwarp; t < tab.total_tasks; t += nwarps) {
     int v = tab.v_lo;
     while (v < tab.v_hi && t >= tab.task_start[v + 1]) ++v;
@@ -221,10 +200,8 @@ __global__ void __launch_bounds__(kMaxThreadsModp) k_modp_prefix(SingleArgs a, P
 #pragma unroll
       for (int j = 0; j < P; ++j) sp += c[j] + 1;
       unsigned long long rank_prefix = 0;
-      if constexpr (kTerms) {
 #pragma unroll
-        for (int j = 0; j < P; ++j) rank_prefix += rank_part(sm.binom, bs, n, c[j], M - j);
-      }
+      for (int j = 0; j < P; ++j) rank_prefix += rank_part(sm.binom, bs, n, c[j], M - j);
 #pragma unroll 1
       for (int k = 0; k < K; ++k) {
         const Mont mp = sm.mont[k];
@@ -234,47 +211,37 @@ __global__ void __launch_bounds__(kMaxThreadsModp) k_modp_prefix(SingleArgs a, P
         bool negp;
         modp_prefix_factor<M, D, CS>(As, c, mp, fa, idx, piv, negp, den);
         negp ^= (sp & 1) != 0;
-        uint32_t inv_den = 0u;
-        if constexpr (kTerms) inv_den = minv(den, mp);  // 0 for a singular prefix: its terms are 0
-        uint32_t* terms = kTerms ? static_cast<uint32_t*>(a.terms) + (size_t)k * a.count : nullptr;
-        const uint32_t S = modp_prefix_leaves<M, D, kTerms>(As, CS, sm.binom, n, v, fa, idx, piv, mp, zb, sub, lp,
-                                                           negp, inv_den, rank_prefix, ts, terms, act);
-        if constexpr (!kTerms) {
-          if (act && den != 0u) acc_fraction(N, Dn, k, S, den, negp, mp);
-        }
+        const uint32_t inv_den = minv(den, mp);  // 0 for a singular prefix: its terms are 0
+        uint32_t* terms = static_cast<uint32_t*>(a.terms) + (size_t)k * a.count;
+        modp_prefix_leaves<M, D>(As, CS, sm.binom, n, v, fa, idx, piv, mp, zb, sub, lp, negp, inv_den, rank_prefix,
+                                 ts, terms, act);
       }
       if constexpr (P > 1) {
         if (r0 + it + 1 < r1) successor<P - 1>(head, v);
       }
     }
   }
-  if constexpr (!kTerms) {
-    uint32_t r[kMaxPrimes];
-    close_fractions(N, Dn, K, sm.mont, r);
-    finish_modp(a, sm, r, K, needed);
-  }
 }
 
 template <int M, int D>
-const void* prefix_kernel(bool terms) {
-  return terms ? reinterpret_cast<const void*>(&k_modp_prefix<M, D, true>)
-               : reinterpret_cast<const void*>(&k_modp_prefix<M, D, false>);
+const void* prefix_kernel() {
+  return reinterpret_cast<const void*>(&k_modp_prefix<M, D>);
 }
 
 }  // namespace
 
-const void* modp_prefix_kernel(int m, int depth, bool terms) {
+const void* modp_prefix_kernel(int m, int depth) {
   switch (m) {
-    case 3: return depth == 2 ? prefix_kernel<3, 2>(terms) : nullptr;
-    case 4: return depth == 3 ? prefix_kernel<4, 3>(terms) : prefix_kernel<4, 2>(terms);
-    case 5: return depth == 3 ? prefix_kernel<5, 3>(terms) : prefix_kernel<5, 2>(terms);
-    case 6: return depth == 3 ? prefix_kernel<6, 3>(terms) : prefix_kernel<6, 2>(terms);
-    case 7: return depth == 3 ? prefix_kernel<7, 3>(terms) : prefix_kernel<7, 2>(terms);
-    case 8: return depth == 3 ? prefix_kernel<8, 3>(terms) : prefix_kernel<8, 2>(terms);
-    case 9: return depth == 3 ? prefix_kernel<9, 3>(terms) : prefix_kernel<9, 2>(terms);
-    case 10: return depth == 3 ? prefix_kernel<10, 3>(terms) : prefix_kernel<10, 2>(terms);
-    case 11: return depth == 3 ? prefix_kernel<11, 3>(terms) : prefix_kernel<11, 2>(terms);
-    case 12: return depth == 3 ? prefix_kernel<12, 3>(terms) : prefix_kernel<12, 2>(terms);
+    case 3: return depth == 2 ? prefix_kernel<3, 2>() : nullptr;
+    case 4: return depth == 3 ? prefix_kernel<4, 3>() : prefix_kernel<4, 2>();
+    case 5: return depth == 3 ? prefix_kernel<5, 3>() : prefix_kernel<5, 2>();
+    case 6: return depth == 3 ? prefix_kernel<6, 3>() : prefix_kernel<6, 2>();
+    case 7: return depth == 3 ? prefix_kernel<7, 3>() : prefix_kernel<7, 2>();
+    case 8: return depth == 3 ? prefix_kernel<8, 3>() : prefix_kernel<8, 2>();
+    case 9: return depth == 3 ? prefix_kernel<9, 3>() : prefix_kernel<9, 2>();
+    case 10: return depth == 3 ? prefix_kernel<10, 3>() : prefix_kernel<10, 2>();
+    case 11: return depth == 3 ? prefix_kernel<11, 3>() : prefix_kernel<11, 2>();
+    case 12: return depth == 3 ? prefix_kernel<12, 3>() : prefix_kernel<12, 2>();
     default: return nullptr;
   }
 }
