@@ -434,10 +434,11 @@ size_t radic_backward_workspace_bytes(int batch, int m, int n);
  * binary64.  d det_R / d A[:, J] = (-1)^(r+s) adj(A[:, J])^T for every
  * column sequence J of Eq. (1): each minor's signed cofactors
  * det(M) inv(M)^T are scatter-added into the gradient columns J.  For
- * m >= 3 the cofactors of all minors of one (m-2)-column prefix are summed
- * in closed form from the prefix's partial-pivot LU (block inverse of the
- * minor); for m <= 2, and for prefixes with an exactly zero pivot, from
- * each minor's own LU.  A: device, batch matrices m x n, row-major with
+ * m >= 3 the cofactors of all minors that begin with the same head of m-G
+ * columns (G = 2..4) are summed in closed form from the head's partial-pivot
+ * LU; heads with an exactly zero pivot are summed without elimination (by
+ * exterior products of the columns), and for m <= 2 every minor has its own
+ * LU.  A: device, batch matrices m x n, row-major with
  * leading dimension lda, matrix b at A + b * stride.  grad_out: device,
  * batch values.  grad_A: device, same layout as A, overwritten.  1 <= m <= 8
  * (m > n gives a zero gradient).  Errors: RADIC_EINVAL, RADIC_EUNSUPPORTED

@@ -13,38 +13,57 @@
 // pivot (singular) takes a slow path that forms its cofactors from
 // (m-1) x (m-1) determinants.
 //
-// For 3 <= m the default kernel shares the work per (m-2)-column prefix, as
-// the forward prefix kernels do, in binary64 or in pairs of binary32.  With the prefix rows T (pivot order) and B
-// (the other two), A = A_TT, W = -A_BT A^{-1}, the Schur complement of a leaf
-// (x, y) is S = [z(x) z(y)], z = x_B + W x_T, det(N) = det(A) det(S) for the
-// row-permuted minor N, and by the block inverse
-//   det(N) N^{-1} = det(A) [[det(S) A^{-1} - A^{-1} X_T adj(S) W, -A^{-1} X_T adj(S)],
-//                           [adj(S) W,                            adj(S)]].
-// Summed over the leaves of the prefix with their signs (column parities
-// folded into z~ = (-1)^col z), every candidate column q receives
-//   alpha (-1)^q [W^T; I] g_q,   g_q = rot(Z_>q - Z_<q),   rot(h) = (h1, -h0),
-// where Z_<q and Z_>q are the sums of z~ over the columns before and after
-// q, and the prefix columns receive alpha [s A^{-1} - A^{-1} Q W | -A^{-1} Q]^T
-// with s = sum over leaves of det[z~_x z~_y] and
-// Q = sum_q (-1)^q x_T(q) g_q^T.  A prefix thus costs O(m^2 (m-2) + k m)
-// operations for its k candidate columns and its C(k, 2) leaves, and scatters
-// m (m - 2 + k) gradient entries.  A prefix with an exactly zero pivot falls
-// back to the per-minor cofactors for its leaves.
+// For 3 <= m the default kernel shares the work per head, the first H = m-G
+// columns (G = 2..4), as the forward prefix kernels do, in binary64 or in
+// pairs of binary32.  With the head's rows T (pivot order) and B (the other G),
+// A = A_TT, W = -A_BT A^{-1}, every later column x has the Schur complement
+// z(x) = x_B + W x_T, and the subtree of the head adds up to alpha L, alpha the
+// signed product of the pivots and L the sum of det[z(x_1) ... z(x_G)] over
+// x_1 < ... < x_G.  L is a polynomial of the z(x), linear in each: with P[S]
+// and R[S] the sums of the determinants of the rows S over all ascending
+// sequences of |S| columns before, and after, column q (column parities folded
+// into z),
+//   g_q,i = dL / dz_i(x_q) = sum over T not holding i of +- P[T] R[rest],
+// the sign that of bringing the rows (T, i, rest) into order.  P and R follow
+// from column to column by one exterior product with z (R by taking z(x_q)
+// out again: R_q = (1 - z) ^ R_{q-1}), G 2^(G-1) multiply-adds each.  Taking
+// columns out keeps the rounding of the larger sums it starts from, so R is
+// built from the last column to the first, kept at two columns on the way, and
+// taken up from there again (with one start alone the gradient's error was
+// 2.1 times that of the sums over two columns, in both arithmetics).  Then
+// column q receives alpha (-1)^q [W^T; I] g_q, and the head's own columns
+// alpha [L A^{-1} - A^{-1} Q W | -A^{-1} Q]^T with Q = sum_q (-1)^q x_T(q) g_q^T.
+// A head thus costs O(k G (2^G + m)) operations for its k later columns,
+// whatever the number C(k, G) of its minors.
 //
-// Gathering those entries: each warp adds into its own gradient tile in
-// shared memory (binary64 or pairs, as the kernel computes), without
-// atomics, and the block adds its warps' tiles in warp order at the end.  The
-// 32 lanes of a warp task hold prefixes with the same last column v, so they
-// share the candidate columns and v: those columns are summed over the warp in
-// registers (a reduce-scatter of the m rows, one lane per entry), v's entries
-// first per lane over the lane's run.  Of the other prefix columns, the ones
-// that change slowly in dictionary order are summed per lane in shared memory
-// and added when the column moves on; the fastest one is added per prefix,
-// lanes with the same column taking turns.  (Atomic binary64 additions to
-// shared memory retry under contention; adding every entry that way, with 32
-// lanes on one column, made them the bulk of the kernel.)
+// What bounds it: the binary64 pipe (a warp instruction takes 16 cycles of an
+// SM, whether or not all its lanes are used) or, in pairs, dependent binary32
+// chains at 8 warps per SM.  G trades the number of heads, C(n-G, m-G),
+// against the cost of a column (bwd_plan).  256 matrices of 6 x 28, binary64:
+// 0.57 ms with G = 4, the pipe 72% busy (6.0 ms with G = 2 and lanes grouped by
+// equal v, the pipe 83% busy).
+//
+// Lanes take heads in colexicographic order (by last column v, then in
+// dictionary order), so that a warp is full whatever the sizes of the groups
+// of equal v, and step through the columns together from the smallest v on;
+// a lane joins in after its own v.
+//
+// Gathering the gradient: each warp adds into its own tile in shared memory
+// (binary64 or pairs, as the kernel computes), without atomics, and the block
+// adds its warps' tiles in warp order at the end.  Later columns are summed
+// over the warp in registers (a reduce-scatter of the m rows, one lane per
+// entry); a head column is added once per distinct column in the warp, or lane
+// by lane where many lanes have columns of their own.  (Atomic binary64
+// additions to shared memory retry under contention; adding every entry that
+// way, with 32 lanes on one column, made them the bulk of the kernel.)
+//
+// A head with an exactly zero pivot has no A^{-1}; its warp sums its subtree
+// without elimination, by the same exterior products over all m rows starting
+// from the determinants of the head's own columns (singular_head), 2^m sums
+// spread over the lanes.
 //
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 
@@ -62,7 +81,9 @@ struct BwdArgs {
   int batch, m, n;
   int chunks;             // blocks per matrix
   unsigned long long total;
-  double* slots;          // batch x chunks x m x n
+  double* slots;          // batch x chunks x m x n (chunks > 1)
+  const double* grad_out;
+  double* grad;           // written directly when chunks == 1
 };
 
 // Full partial-pivot LU with multipliers stored below the diagonal; idx[s] is
@@ -249,38 +270,6 @@ __global__ void __launch_bounds__(kBwdThreads) k_backward(BwdArgs a) {
   for (int idx = threadIdx.x; idx < M * n; idx += blockDim.x) slot[idx] = G[idx];
 }
 
-// Signed cofactors of one minor read from the binary64 matrix in global
-// memory (row stride lda), added into the gradient tile G.
-template <int M>
-__device__ __noinline__ void minor_cofactors_scatter_global(const double* Ab, long long lda, const int (&c)[M],
-                                                            double* G, int n) {
-  constexpr int CSG = ColStride<double, M>::value;
-  double col[M * CSG];
-  for (int j = 0; j < M; ++j)
-    for (int i = 0; i < CSG; ++i) col[j * CSG + i] = (i < M) ? Ab[(long long)i * lda + c[j]] : 0.0;
-  int cl[M];
-  for (int j = 0; j < M; ++j) cl[j] = j;
-  double mm[M][M];
-  for (int j = 0; j < M; ++j)
-    for (int i = 0; i < M; ++i) mm[i][j] = col[j * CSG + i];
-  int idx[M];
-  bool zp;
-  const double det = lu_full<M>(mm, idx, zp);
-  const double sgn = sign_negative<M>(c) ? -1.0 : 1.0;
-  if (!zp) {
-    double B[M][M];
-    inverse_factors<M>(mm, B);
-    const double s = sgn * det;
-    for (int sl = 0; sl < M; ++sl)
-      for (int j = 0; j < M; ++j) atomicAdd(G + idx[sl] * n + c[j], s * B[j][sl]);
-  } else {
-    double cof[M][M];
-    cofactors_slow<M>(col, CSG, cl, cof);
-    for (int i = 0; i < M; ++i)
-      for (int j = 0; j < M; ++j) atomicAdd(G + i * n + c[j], sgn * cof[i][j]);
-  }
-}
-
 __device__ __forceinline__ bool pivot_greater(double x, double y) { return mag_key(x) > mag_key(y); }
 __device__ __forceinline__ bool pivot_greater(ff x, ff y) { return fabsf(x.hi) > fabsf(y.hi); }
 __device__ __forceinline__ bool is_zero(double x) { return x == 0.0; }
@@ -396,299 +385,474 @@ __device__ __forceinline__ void unpermute(const T (&x)[M], const int (&idx)[M], 
   }
 }
 
+// Adds u[0..M-1] to column `key` of the warp's tile for the lanes with key >=
+// 0: one warp sum per distinct column where they are few, turns otherwise (a
+// warp sum takes about three times as long as a turn).
 template <typename T, int M>
-__global__ void __launch_bounds__(kBwdThreads) k_backward_prefix(BwdArgs a, PrefixTable tab) {
-  constexpr int D = 2, P = M - D;
-  // head positions 0 .. P-3 change slowly in dictionary order and are summed
-  // per lane in shared memory (NS of them); position P-2 changes with every
-  // prefix and is added directly; column v is the same for the whole warp
-  constexpr int NS = P > 2 ? P - 2 : 0;
+__device__ __forceinline__ void warp_add_head_column(T* tile, int n, int key, const T (&u)[M], int lane) {
+  const unsigned grp = __match_any_sync(kFull, key);
+  const unsigned first = __ballot_sync(kFull, key >= 0 && lane == __ffs(grp) - 1);
+  const unsigned rounds = __reduce_max_sync(kFull, key >= 0 ? (unsigned)__popc(grp) : 0u);
+  if (3u * __popc(first) > rounds) {
+    warp_tile_add<T, M>(tile, n, key, u, lane);
+    return;
+  }
+  for (unsigned todo = first; todo; todo &= todo - 1) {
+    const int col = __shfl_sync(kFull, key, __ffs(todo) - 1);
+    T w[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) w[i] = key == col ? u[i] : T(0);
+    warp_add_column<T, M>(w, tile + col, n, lane);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Exterior sums over sets of G rows (see the head of this file), unrolled at
+// compile time.  Entry S of an array belongs to the rows in the bit set S;
+// entry 0 (the empty set, 1) is never stored.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int bits_of(unsigned x) { return x ? static_cast<int>(x & 1u) + bits_of(x >> 1) : 0; }
+// Parity of the order (T, i, U): pairs out of order.
+__host__ __device__ constexpr bool odd_order(unsigned T, int i, unsigned U) {
+  int inv = bits_of(T >> (i + 1)) + bits_of(U & ((1u << i) - 1u));
+  for (unsigned r = U; r; r &= r - 1) {
+    int u = 0;
+    while (!((r >> u) & 1u)) ++u;
+    inv += bits_of(T >> (u + 1));
+  }
+  return inv & 1;
+}
+
+template <typename T>
+__device__ __forceinline__ T signed_of(bool neg, T x) {
+  return neg ? -x : x;
+}
+
+// P[S] += sum over i in S of +- z_i P[S without i], z appended as the last
+// column, for the sets of at most MAXS rows from SET down to 1.
+template <typename T, int G, int MAXS, int SET>
+__device__ __forceinline__ void append_column(T (&P)[1 << G], const T (&z)[G]) {
+  if constexpr (SET >= 1) {
+    constexpr int size = bits_of(SET);
+    if constexpr (size <= MAXS) {
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if ((SET >> i) & 1) {
+          const bool neg = (size - 1 - bits_of(SET & ((1 << i) - 1))) & 1;
+          if constexpr (size == 1) P[SET] = P[SET] + z[i];
+          else P[SET] = fma(signed_of(neg, z[i]), P[SET ^ (1 << i)], P[SET]);
+        }
+      }
+    }
+    append_column<T, G, MAXS, SET - 1>(P, z);
+  }
+}
+
+// R <- (1 + z) ^ R (kAdd: z becomes the first column of R's sequences) or
+// (1 - z) ^ R (takes the first column z out again).
+template <typename T, int G, bool kAdd, int MAXS, int SET>
+__device__ __forceinline__ void first_column(T (&R)[1 << G], const T (&z)[G]) {
+  if constexpr (SET >= 1) {
+    constexpr int size = bits_of(SET);
+    if constexpr (size <= MAXS) {
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if ((SET >> i) & 1) {
+          const bool neg = (bits_of(SET & ((1 << i) - 1)) & 1) != (kAdd ? 0 : 1);
+          if constexpr (size == 1) R[SET] = R[SET] + signed_of(neg, z[i]);
+          else R[SET] = fma(signed_of(neg, z[i]), R[SET ^ (1 << i)], R[SET]);
+        }
+      }
+    }
+    first_column<T, G, kAdd, MAXS, SET - 1>(R, z);
+  }
+}
+
+// g_I: sum over the sets SET not holding I of +- P[SET] R[the other rows].
+template <typename T, int G, int I, int SET>
+__device__ __forceinline__ void contract_row(const T (&P)[1 << G], const T (&R)[1 << G], T& g) {
+  if constexpr (SET < (1 << G)) {
+    if constexpr (!((SET >> I) & 1)) {
+      constexpr int rest = ((1 << G) - 1) ^ SET ^ (1 << I);
+      constexpr bool neg = odd_order(SET, I, rest);
+      if constexpr (SET == 0) g = signed_of(neg, R[rest]);
+      else if constexpr (rest == 0) g = g + signed_of(neg, P[SET]);
+      else g = fma(signed_of(neg, P[SET]), R[rest], g);
+    }
+    contract_row<T, G, I, SET + 1>(P, R, g);
+  }
+}
+template <typename T, int G, int I = 0>
+__device__ __forceinline__ void contract(const T (&P)[1 << G], const T (&R)[1 << G], T (&g)[G]) {
+  if constexpr (I < G) {
+    contract_row<T, G, I, 0>(P, R, g[I]);
+    contract<T, G, I + 1>(P, R, g);
+  }
+}
+
+// Gradient of a head's subtree without elimination, by the whole warp, in
+// binary64 from the matrix in global memory: the same sums over sets of all M
+// rows, a prefix sum V that starts from the determinants of the head's columns
+// instead of 1, and suffix sums R over the later columns.  Serves heads with
+// an exactly zero pivot.  scratch: 2^(M+1) words of shared memory; G: the
+// block's gradient tile (shared-memory atomics).
+template <int M, int GD>
+__device__ __noinline__ void singular_head(const double* Ab, long long lda, const int (&c)[M - GD], int n,
+                                           double* scratch, double* G, int lane) {
+  constexpr int H = M - GD, NS = 1 << M;
+  double* V = scratch;
+  double* R = scratch + NS;
+  auto entry = [&](int i, int col) {  // column parity of Eq. (1) folded in
+    const double x = Ab[(long long)i * lda + col];
+    return (col & 1) ? -x : x;
+  };
+  // E <- E + E ^ x (front: (1 - x) ^ E) for the sets of lo..hi rows, largest first
+  auto wedge = [&](double* E, int col, int lo, int hi, bool front) {
+    for (int size = hi; size >= lo; --size) {
+      for (int S = lane; S < NS; S += 32) {
+        if (__popc(S) != size) continue;
+        double acc = E[S];
+        int pos = 0;
+        for (int i = 0; i < M; ++i) {
+          if (!((S >> i) & 1)) continue;
+          const bool neg = front ? !(pos & 1) : ((size - 1 - pos) & 1);
+          const double t = entry(i, col) * E[S ^ (1 << i)];
+          acc += neg ? -t : t;
+          ++pos;
+        }
+        E[S] = acc;
+      }
+      __syncwarp();
+    }
+  };
+  // sum over the sets T without row i of +- V[T] R[rest], for every row i,
+  // into column `col` of the tile
+  auto scatter = [&](int col, bool neg) {
+    for (int i = 0; i < M; ++i) {
+      double s = 0.0;
+      for (int T = lane; T < NS; T += 32) {
+        if ((T >> i) & 1) continue;
+        const int rest = (NS - 1) ^ T ^ (1 << i);
+        int inv = __popc(T >> (i + 1)) + __popc(rest & ((1 << i) - 1));
+        for (int u = 0; u < M; ++u)
+          if ((rest >> u) & 1) inv += __popc(T >> (u + 1));
+        const double t = V[T] * R[rest];
+        s += (inv & 1) ? -t : t;
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+      if (lane == 0) atomicAdd(G + i * n + col, neg ? -s : s);
+    }
+    __syncwarp();
+  };
+  auto unit = [&](double* E) {
+    for (int S = lane; S < NS; S += 32) E[S] = S == 0 ? 1.0 : 0.0;
+    __syncwarp();
+  };
+  const bool common = (M * (M + 1) / 2 + M) & 1;  // (-1)^(r+s) without the column parities
+  // suffix sums over all later columns, sets of up to GD rows
+  unit(R);
+  for (int col = c[H - 1] + 1; col < n; ++col) wedge(R, col, 1, GD, false);
+  // head column j: the determinants of the other head columns (sets of H-1
+  // rows) against the sums over GD columns; column j moves past H-1-j columns
+  for (int j = 0; j < H; ++j) {
+    unit(V);
+    int size = 0;
+    for (int t = 0; t < H; ++t) {
+      if (t == j) continue;
+      wedge(V, c[t], 1, ++size, false);
+    }
+    for (int S = lane; S < NS; S += 32)
+      if (__popc(S) != H - 1) V[S] = 0.0;
+    __syncwarp();
+    scatter(c[j], common ^ ((c[j] & 1) != 0) ^ (((H - 1 - j) & 1) != 0));
+  }
+  // later columns: V starts from the head's own determinants
+  unit(V);
+  for (int t = 0; t < H; ++t) wedge(V, c[t], 1, t + 1, false);
+  for (int S = lane; S < NS; S += 32)
+    if (__popc(S) != H) V[S] = 0.0;
+  __syncwarp();
+  for (int col = c[H - 1] + 1; col < n; ++col) {
+    wedge(R, col, 1, GD, true);
+    scatter(col, common ^ ((col & 1) != 0));
+    wedge(V, col, H + 1, M - 1, false);
+  }
+}
+
+// Shared-memory layout of the head kernel.
+template <typename T>
+struct BwdSmem {
+  uint64_t* binom;
+  T* As;
+  double* tile0;    // tile of the singular heads
+  T* tiles;         // one m x n tile per warp
+  double* scratch;  // 2^(m+1) words per warp
+  T* kept;          // R at two columns, 2^G - 2 sums each, lane by lane
+  size_t bytes;
+  __host__ __device__ BwdSmem(unsigned char* base, int n, int m, int G, int warps) {
+    size_t off = 0;
+    auto take = [&](size_t b) {
+      const size_t o = off;
+      off += (b + 15) / 16 * 16;
+      return o;
+    };
+    binom = reinterpret_cast<uint64_t*>(base + take((size_t)(n + 1) * (m + 1) * 8));
+    As = reinterpret_cast<T*>(base + take((size_t)n * ((m + 1) / 2 * 2) * 8));
+    tile0 = reinterpret_cast<double*>(base + take((size_t)m * n * 8));
+    tiles = reinterpret_cast<T*>(base + take((size_t)warps * m * n * 8));
+    scratch = reinterpret_cast<double*>(base + take((size_t)warps * (16u << m)));
+    kept = reinterpret_cast<T*>(base + take((size_t)2 * ((1 << G) - 2) * warps * 32 * 8));
+    bytes = off;
+  }
+};
+
+template <typename T, int M, int G>
+__global__ void __launch_bounds__(kBwdThreads, 2) k_backward_heads(BwdArgs a) {
+  constexpr int H = M - G, FULL = (1 << G) - 1;
   constexpr int CS = ColStride<T, M>::value;
+  static_assert(sizeof(T) == 8 && CS == (M + 1) / 2 * 2, "layout of BwdSmem");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n = a.n;
+  const int n = a.n, bs = M + 1;
   const int b = blockIdx.y, chunk = blockIdx.x;
-  uint64_t* binom = reinterpret_cast<uint64_t*>(smem_raw);
-  size_t off = ((size_t)(n + 1) * (M + 1) * 8 + 15) / 16 * 16;
-  T* As = reinterpret_cast<T*>(smem_raw + off);
-  off += ((size_t)n * CS * sizeof(T) + 15) / 16 * 16;
-  double* G = reinterpret_cast<double*>(smem_raw + off);  // M x n tile of the singular-prefix path
-  off += ((size_t)M * n * 8 + 15) / 16 * 16;
-  const ZBuf<T, D> zb(smem_raw + off, threadIdx.x, blockDim.x, n - M + D);
-  off += (zbuf_bytes(n - M + D, blockDim.x, D, 8) + 15) / 16 * 16;
-  T* Hacc = reinterpret_cast<T*>(smem_raw + off) + threadIdx.x;  // [NS][M] per lane, lane-strided
-  off += (size_t)NS * M * blockDim.x * sizeof(T);
-  T* Gall = reinterpret_cast<T*>(smem_raw + off);  // one M x n tile per warp
-  build_binom(binom, n, M);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+  const BwdSmem<T> sm(smem_raw, n, M, G, wpb);
+  build_binom(sm.binom, n, M);
   const double* Ab = a.A + (long long)b * a.stride;
   for (int idx = threadIdx.x; idx < n * CS; idx += blockDim.x) {
-    const int j = idx / CS, i = idx - j * CS;
-    As[idx] = (i < M) ? to_elem<T>(Ab[(long long)i * a.lda + j]) : T(0);
+    const int i = idx / n, j = idx - i * n;  // rows of A are contiguous
+    sm.As[j * CS + i] = (i < M) ? to_elem<T>(Ab[(long long)i * a.lda + j]) : T(0);
   }
-  for (int idx = threadIdx.x; idx < M * n; idx += blockDim.x) G[idx] = 0.0;
-  for (int idx = threadIdx.x; idx < (int)(blockDim.x >> 5) * M * n; idx += blockDim.x) Gall[idx] = T(0);
+  for (int idx = threadIdx.x; idx < M * n; idx += blockDim.x) sm.tile0[idx] = 0.0;
+  for (int idx = threadIdx.x; idx < wpb * M * n; idx += blockDim.x) sm.tiles[idx] = T(0);
   __syncthreads();
+  const T* As = sm.As;
+  T* Gw = sm.tiles + (size_t)warp * M * n;
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  const int bs = M + 1;
-  const int hs = blockDim.x;
-  T* Gw = Gall + (size_t)warp * M * n;  // stride between a lane's accumulator entries
-  for (unsigned long long t = (unsigned long long)chunk * wpb + warp; t < tab.total_tasks;
+  // heads in colexicographic order: those with last column v are the ranks
+  // C(v, H) .. C(v+1, H) - 1
+  const unsigned long long heads = sm.binom[(n - G) * bs + H];
+  const unsigned long long tasks = (heads + 31) / 32;
+  for (unsigned long long t = (unsigned long long)chunk * wpb + warp; t < tasks;
        t += (unsigned long long)a.chunks * wpb) {
-    // everything up to the step loop is the same for the 32 lanes of the task
-    int v = tab.v_lo;
-    while (v < tab.v_hi && t >= tab.task_start[v + 1]) ++v;
-    const unsigned long long runlen = tab.run[v], cnt = tab.count[v];
-    const unsigned long long r0 = (t - tab.task_start[v]) * 32ull * runlen + (unsigned long long)lane * runlen;
-    const unsigned long long r1 = min(r0 + runlen, cnt);
-    const bool ever = r0 < r1;  // true for lane 0: a task starts below cnt
-    constexpr int H = P > 1 ? P - 1 : 1;
-    int head[H];
-    if constexpr (P > 1) unrank<P - 1>(ever ? r0 : cnt - 1, v, binom, bs, head);
-    const int k = n - 1 - v;
-    T vacc[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) vacc[i] = T(0);
-    int hcol[NS > 0 ? NS : 1];
-#pragma unroll
-    for (int p = 0; p < NS; ++p) {
-      hcol[p] = head[p];
-#pragma unroll
-      for (int i = 0; i < M; ++i) Hacc[(p * M + i) * hs] = T(0);
+    const bool live = t * 32 + lane < heads;
+    const unsigned long long r = live ? t * 32 + lane : heads - 1;
+    int v = H - 1, hi = n - G;  // C(v, H) <= r < C(hi, H)
+    while (hi - v > 1) {
+      const int mid = (v + hi) / 2;
+      if (sm.binom[mid * bs + H] <= r) v = mid;
+      else hi = mid;
     }
-    // lanes past their run repeat their last prefix with zero weight, so that
-    // the whole warp takes every step (the column sums exchange registers)
-    for (unsigned long long st = 0; st < runlen; ++st) {
-      const unsigned long long r = r0 + st;
-      const bool live = r < r1;
-      int c[P];
+    int c[H];
+    c[H - 1] = v;
+    if constexpr (H > 1) {
+      int head[H - 1];
+      unrank<H - 1>(r - sm.binom[v * bs + H], v, sm.binom, bs, head);
 #pragma unroll
-      for (int j = 0; j < P - 1; ++j) c[j] = head[j];
-      c[P - 1] = v;
-      // factor the M x P prefix: partial pivoting, L \ U packed in fa
-      T fa[M][P];
+      for (int j = 0; j < H - 1; ++j) c[j] = head[j];
+    }
+    const int col0 = __shfl_sync(kFull, v, 0) + 1;  // the smallest v is lane 0's
+    // factor the M x H head: partial pivoting, L \ U packed in fa
+    T fa[M][H];
 #pragma unroll
-      for (int j = 0; j < P; ++j)
+    for (int j = 0; j < H; ++j)
 #pragma unroll
-        for (int i = 0; i < M; ++i) fa[i][j] = As[c[j] * CS + i];
-      int idx[M];
+      for (int i = 0; i < M; ++i) fa[i][j] = As[c[j] * CS + i];
+    int idx[M];
 #pragma unroll
-      for (int i = 0; i < M; ++i) idx[i] = i;
-      bool neg = false, zp = false;
-      T prod = T(1);
+    for (int i = 0; i < M; ++i) idx[i] = i;
+    bool neg = false, zp = false;
+    T prod = T(1);
 #pragma unroll
-      for (int kk = 0; kk < P; ++kk) {
+    for (int kk = 0; kk < H; ++kk) {
 #pragma unroll
-        for (int i = kk + 1; i < M; ++i) {
-          const bool sw = pivot_greater(fa[i][kk], fa[kk][kk]);
+      for (int i = kk + 1; i < M; ++i) {
+        const bool sw = pivot_greater(fa[i][kk], fa[kk][kk]);
 #pragma unroll
-          for (int j = 0; j < P; ++j) {
-            const T x = fa[kk][j], y = fa[i][j];
-            fa[kk][j] = sw ? y : x;
-            fa[i][j] = sw ? x : y;
-          }
-          const int ik = idx[kk], ii = idx[i];
-          idx[kk] = sw ? ii : ik;
-          idx[i] = sw ? ik : ii;
-          neg ^= sw;
+        for (int j = 0; j < H; ++j) {
+          const T x = fa[kk][j], y = fa[i][j];
+          fa[kk][j] = sw ? y : x;
+          fa[i][j] = sw ? x : y;
         }
-        const T piv = fa[kk][kk];
-        zp |= is_zero(piv);
-        prod *= piv;
-        const T rr = rcp_t(piv);
-#pragma unroll
-        for (int i = kk + 1; i < M; ++i) {
-          const T l = fa[i][kk] * rr;
-          fa[i][kk] = l;
-#pragma unroll
-          for (int j = kk + 1; j < P; ++j) fa[i][j] = fma(-l, fa[kk][j], fa[i][j]);
-        }
+        const int ik = idx[kk], ii = idx[i];
+        idx[kk] = sw ? ii : ik;
+        idx[i] = sw ? ik : ii;
+        neg ^= sw;
       }
-      if (live && zp) {  // singular prefix: per-minor cofactors of its leaves
-        for (int x = v + 1; x < n; ++x)
-          for (int y = x + 1; y < n; ++y) {
-            int cm[M];
-            for (int j = 0; j < P; ++j) cm[j] = c[j];
-            cm[P] = x;
-            cm[P + 1] = y;
-            minor_cofactors_scatter_global<M>(Ab, a.lda, cm, G, n);
-          }
+      const T piv = fa[kk][kk];
+      zp |= is_zero(piv);
+      prod *= piv;
+      const T rr = rcp_t(piv);
+#pragma unroll
+      for (int i = kk + 1; i < M; ++i) {
+        const T l = fa[i][kk] * rr;
+        fa[i][kk] = l;
+#pragma unroll
+        for (int j = kk + 1; j < H; ++j) fa[i][j] = fma(-l, fa[kk][j], fa[i][j]);
       }
-      // below, a singular or repeated prefix runs with non-finite or unwanted
-      // values that `use` replaces by zeros
-      const bool use = live && !zp;
-      // W = -L21 L11^{-1} (D x P) and Ainv = U11^{-1} L11^{-1} (P x P)
-      T W[D][P];
+    }
+    for (unsigned sing = __ballot_sync(kFull, live && zp); sing; sing &= sing - 1) {
+      int cs[H];
 #pragma unroll
-      for (int d = 0; d < D; ++d) {
+      for (int j = 0; j < H; ++j) cs[j] = __shfl_sync(kFull, c[j], __ffs(sing) - 1);
+      singular_head<M, G>(Ab, a.lda, cs, n, sm.scratch + (size_t)warp * (2u << M), sm.tile0, lane);
+    }
+    // below, a singular or repeated head runs with non-finite or unwanted
+    // values that `use` replaces by zeros
+    const bool use = live && !zp;
+    // W = -L21 L11^{-1} (G x H) and Ainv = U11^{-1} L11^{-1} (H x H)
+    T W[G][H], Ai[H][H];
 #pragma unroll
-        for (int j = P - 1; j >= 0; --j) {
-          T sum = -fa[P + d][j];
+    for (int d = 0; d < G; ++d) {
 #pragma unroll
-          for (int i = j + 1; i < P; ++i) sum = fma(-W[d][i], fa[i][j], sum);
-          W[d][j] = sum;
-        }
+      for (int j = H - 1; j >= 0; --j) {
+        T sum = -fa[H + d][j];
+#pragma unroll
+        for (int i = j + 1; i < H; ++i) sum = fma(-W[d][i], fa[i][j], sum);
+        W[d][j] = sum;
       }
-      T Ai[P][P];
-      {
-        T top[P][P];
+    }
+    {
+      T top[H][H];
 #pragma unroll
-        for (int i = 0; i < P; ++i)
+      for (int i = 0; i < H; ++i)
 #pragma unroll
-          for (int j = 0; j < P; ++j) top[i][j] = fa[i][j];
-        inverse_factors<P, T>(top, Ai);
+        for (int j = 0; j < H; ++j) top[i][j] = fa[i][j];
+      inverse_factors<H, T>(top, Ai);
+    }
+    int sp = M * (M + 1) / 2 + G;
+#pragma unroll
+    for (int j = 0; j < H; ++j) sp += c[j] + 1;
+    const T alpha = ((sp & 1) != neg) ? -prod : prod;
+    auto schur = [&](int col, T (&z)[G]) {
+      prefix_column<T, M, G>(As + col * CS, W, idx, z);
+      if (col & 1) {
+#pragma unroll
+        for (int d = 0; d < G; ++d) z[d] = -z[d];
       }
-      int sp = M * (M + 1) / 2 + D;
+    };
+    // pass 1: the sums over all later columns; R[FULL] = L
+    T R[1 << G], P[1 << G];
 #pragma unroll
-      for (int j = 0; j < P; ++j) sp += c[j] + 1;
-      const T alpha = ((sp & 1) != neg) ? -prod : prod;
-      // pass 1: z~ of every candidate column, their sum, and s
-      T zt0 = T(0), zt1 = T(0), ssum = T(0);
-      for (int q = 0; q < k; ++q) {
-        const int col = v + 1 + q;
-        T z[D];
-        prefix_column<T, M, D>(As + col * CS, W, idx, z);
-        if (col & 1) {
-          z[0] = -z[0];
-          z[1] = -z[1];
-        }
-        ssum = fma(zt0, z[1], fma(-zt1, z[0], ssum));  // det[Z_<q, z~_q]
-        zt0 += z[0];
-        zt1 += z[1];
-        zb.put(q, z);
+    for (int S = 0; S <= FULL; ++S) R[S] = P[S] = T(0);
+    // kept at third points of the warp's columns
+    const int third = (n - col0 + 2) / 3, keep1 = col0 + third, keep2 = keep1 + third;
+    T* kept = sm.kept + threadIdx.x;
+    for (int col = n - 1; col >= col0; --col) {
+      if (col > v) {
+        T z[G];
+        schur(col, z);
+        first_column<T, G, true, G, FULL>(R, z);
       }
-      // the gradient of candidate column q at pivot slot r is
-      // (-1)^q alpha ([W^T; I] g_q)[r]; Ca, Cb hold [W^T; I] in row order
-      T Ca[M], Cb[M];
-      {
-        T ca[M], cb[M];
+      if (col == keep1 || col == keep2) {
 #pragma unroll
-        for (int r = 0; r < M; ++r) {
-          ca[r] = r < P ? W[0][r < P ? r : 0] : (r == P ? T(1) : T(0));
-          cb[r] = r < P ? W[1][r < P ? r : 0] : (r == P + 1 ? T(1) : T(0));
-        }
-        unpermute<T, M>(ca, idx, Ca);
-        unpermute<T, M>(cb, idx, Cb);
+        for (int S = 1; S < FULL; ++S) kept[((col == keep1 ? 0 : FULL - 1) + S - 1) * kBwdThreads] = R[S];
       }
-      // pass 2: candidate-column gradients (summed over the warp) and Q
-      T Q[P][D];
+    }
+    const T L = R[FULL];
+    // pass 2: gradients of the later columns (summed over the warp) and Q
+    T Q[H][G];
 #pragma unroll
-      for (int i = 0; i < P; ++i) Q[i][0] = Q[i][1] = T(0);
-      T zp0 = T(0), zp1 = T(0);
-      auto column = [&](int q, T (&val)[M]) {
-        const int col = v + 1 + q;
-        T z[D];
-        zb.get(q, z);
-        const T h0 = zt0 - (zp0 + zp0) - z[0], h1 = zt1 - (zp1 + zp1) - z[1];
-        const T g0 = h1, g1 = -h0;  // rot(Z_>q - Z_<q)
-        zp0 += z[0];
-        zp1 += z[1];
-        const T sc = (col & 1) ? -alpha : alpha;
+    for (int i = 0; i < H; ++i)
 #pragma unroll
-        for (int i = 0; i < M; ++i) val[i] = use ? sc * fma(Ca[i], g0, Cb[i] * g1) : T(0);
+      for (int d = 0; d < G; ++d) Q[i][d] = T(0);
+    auto column = [&](int col, T (&val)[M]) {
+#pragma unroll
+      for (int i = 0; i < M; ++i) val[i] = T(0);
+      if (col == keep1 || col == keep2) {
+#pragma unroll
+        for (int S = 1; S < FULL; ++S) R[S] = kept[((col == keep1 ? 0 : FULL - 1) + S - 1) * kBwdThreads];
+      }
+      if (col > v) {
+        T z[G], g[G];
+        schur(col, z);
+        first_column<T, G, false, G - 1, FULL>(R, z);
+        contract<T, G>(P, R, g);
+        append_column<T, G, G - 1, FULL>(P, z);
         const T* xc = As + col * CS;
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
+        for (int i = 0; i < H; ++i) {
           const T xt = (col & 1) ? -xc[idx[i]] : xc[idx[i]];
-          Q[i][0] = fma(xt, g0, Q[i][0]);
-          Q[i][1] = fma(xt, g1, Q[i][1]);
-        }
-      };
-      if constexpr (std::is_same<T, ff>::value) {
-        // pairs: one column per warp sum (the column body is long; inlining
-        // it twice measured slower, with instruction-fetch stalls)
-        for (int q = 0; q < k; ++q) {
-          T va[M];
-          column(q, va);
-          warp_add_column<T, M>(va, Gw + v + 1 + q, n, lane);
-        }
-      } else {
-        for (int q = 0; q < k; q += 2) {  // binary64: two columns per warp sum
-          const bool two = q + 1 < k;
-          T va[M], vb[M];
-          column(q, va);
-          if (two) {
-            column(q + 1, vb);
-          } else {
 #pragma unroll
-            for (int i = 0; i < M; ++i) vb[i] = T(0);
-          }
-          warp_add_columns2<T, M>(va, vb, Gw + v + 1 + q, n, lane, two);
+          for (int d = 0; d < G; ++d) Q[i][d] = fma(xt, g[d], Q[i][d]);
         }
+        const T sc = (col & 1) ? -alpha : alpha;
+        T w[M];
+#pragma unroll
+        for (int d = 0; d < G; ++d) {
+          g[d] = use ? sc * g[d] : T(0);
+          w[H + d] = g[d];
+        }
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+          T s = use ? W[0][i] * g[0] : T(0);
+#pragma unroll
+          for (int d = 1; d < G; ++d) s = use ? fma(W[d][i], g[d], s) : T(0);
+          w[i] = s;
+        }
+        unpermute<T, M>(w, idx, val);
       }
-      // prefix columns: alpha [s Ainv - Ainv Q W | -Ainv Q]^T, formed in row
-      // order: with a = (Ainv row tt, 0, 0) in pivot order, row idx[r] of
-      // column c[tt] receives alpha (s a[r] - (Ainv Q)[tt] . [W^T; I][r])
-#pragma unroll
-      for (int tt = 0; tt < P; ++tt) {
-        T R0 = T(0), R1 = T(0);  // (Ainv Q)[tt][:]
-#pragma unroll
-        for (int u = 0; u < P; ++u) {
-          R0 = fma(Ai[tt][u], Q[u][0], R0);
-          R1 = fma(Ai[tt][u], Q[u][1], R1);
-        }
-        T ai[M], air[M];
-#pragma unroll
-        for (int r = 0; r < M; ++r) ai[r] = r < P ? Ai[tt][r < P ? r : 0] : T(0);
-        unpermute<T, M>(ai, idx, air);
-        T u[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) u[i] = alpha * (ssum * air[i] - fma(R0, Ca[i], R1 * Cb[i]));
-        if (tt == P - 1) {
-#pragma unroll
-          for (int i = 0; i < M; ++i) vacc[i] += use ? u[i] : T(0);
-        } else if (tt < NS) {
-#pragma unroll
-          for (int i = 0; i < M; ++i) {
-            T& h = Hacc[(tt * M + i) * hs];
-            h += use ? u[i] : T(0);
-          }
+    };
+    if constexpr (std::is_same<T, ff>::value) {
+      // pairs: one column per warp sum (the column body is long; inlining it
+      // twice measured slower, with instruction-fetch stalls)
+      for (int col = col0; col < n; ++col) {
+        T va[M];
+        column(col, va);
+        warp_add_column<T, M>(va, Gw + col, n, lane);
+      }
+    } else {
+      for (int col = col0; col < n; col += 2) {  // binary64: two columns per warp sum
+        const bool two = col + 1 < n;
+        T va[M], vb[M];
+        column(col, va);
+        if (two) {
+          column(col + 1, vb);
         } else {
-          warp_tile_add<T, M>(Gw, n, use ? c[tt] : -1, u, lane);
+#pragma unroll
+          for (int i = 0; i < M; ++i) vb[i] = T(0);
         }
-      }
-      if constexpr (P > 1) {
-        const bool adv = r + 1 < r1;
-        if (adv) successor<P - 1>(head, v);
-#pragma unroll
-        for (int p = 0; p < NS; ++p) {
-          const bool moved = adv && head[p] != hcol[p];
-          if (__any_sync(kFull, moved)) {  // a slow head column moved on: add its sum
-            T u[M];
-#pragma unroll
-            for (int i = 0; i < M; ++i) u[i] = Hacc[(p * M + i) * hs];
-            warp_tile_add<T, M>(Gw, n, moved ? hcol[p] : -1, u, lane);
-            if (moved) {
-#pragma unroll
-              for (int i = 0; i < M; ++i) Hacc[(p * M + i) * hs] = T(0);
-              hcol[p] = head[p];
-            }
-          }
-        }
+        warp_add_columns2<T, M>(va, vb, Gw + col, n, lane, two);
       }
     }
-    // the task's sums of column v and of the slow head columns
-    warp_add_column<T, M>(vacc, Gw + v, n, lane);
+    // head columns: alpha [L Ainv - Ainv Q W | -Ainv Q]^T, in pivot order row
+    // r of column c[tt]: alpha (L Ainv[tt][r] - (Ainv Q)[tt] . W[.][r]), and
+    // -alpha (Ainv Q)[tt][d] for the rows H + d
 #pragma unroll
-    for (int p = 0; p < NS; ++p) {
-      T u[M];
+    for (int tt = 0; tt < H; ++tt) {
+      T q[G];
 #pragma unroll
-      for (int i = 0; i < M; ++i) u[i] = Hacc[(p * M + i) * hs];
-      const int c0 = __shfl_sync(kFull, hcol[p], 0);
-      if (__all_sync(kFull, !ever || hcol[p] == c0)) {
-        warp_add_column<T, M>(u, Gw + c0, n, lane);
-      } else {
-        warp_tile_add<T, M>(Gw, n, ever ? hcol[p] : -1, u, lane);
+      for (int d = 0; d < G; ++d) {
+        q[d] = Ai[tt][0] * Q[0][d];
+#pragma unroll
+        for (int u = 1; u < H; ++u) q[d] = fma(Ai[tt][u], Q[u][d], q[d]);
       }
+      T w[M], u[M];
+#pragma unroll
+      for (int r2 = 0; r2 < H; ++r2) {
+        T s = L * Ai[tt][r2];
+#pragma unroll
+        for (int d = 0; d < G; ++d) s = fma(-q[d], W[d][r2], s);
+        w[r2] = use ? alpha * s : T(0);
+      }
+#pragma unroll
+      for (int d = 0; d < G; ++d) w[H + d] = use ? -(alpha * q[d]) : T(0);
+      unpermute<T, M>(w, idx, u);
+      warp_add_head_column<T, M>(Gw, n, use ? c[tt] : -1, u, lane);
     }
   }
   __syncthreads();
-  // the block's tile: the singular-prefix entries plus the warps' tiles in
+  // the block's tile: the singular heads' entries plus the warps' tiles in
   // warp order
-  double* slot = a.slots + ((size_t)b * a.chunks + chunk) * (size_t)M * n;
   for (int idx = threadIdx.x; idx < M * n; idx += blockDim.x) {
-    double sum = G[idx];
-    for (int w = 0; w < wpb; ++w) sum += to_double(Gall[(size_t)w * M * n + idx]);
-    slot[idx] = sum;
+    double sum = sm.tile0[idx];
+    for (int w = 0; w < wpb; ++w) sum += to_double(sm.tiles[(size_t)w * M * n + idx]);
+    if (a.chunks == 1) {
+      const int i = idx / n, j = idx - i * n;
+      a.grad[(long long)b * a.stride + (long long)i * a.lda + j] = sum * a.grad_out[b];
+    } else {
+      a.slots[((size_t)b * a.chunks + chunk) * (size_t)M * n + idx] = sum;
+    }
   }
 }
 
@@ -708,87 +872,77 @@ __global__ void k_backward_reduce(const double* slots, int batch, int m, int n, 
 }
 
 const void* bwd_kernel(int m) {
-  switch (m) {
-    case 1: return reinterpret_cast<const void*>(&k_backward<1>);
-    case 2: return reinterpret_cast<const void*>(&k_backward<2>);
-    case 3: return reinterpret_cast<const void*>(&k_backward<3>);
-    case 4: return reinterpret_cast<const void*>(&k_backward<4>);
-    case 5: return reinterpret_cast<const void*>(&k_backward<5>);
-    case 6: return reinterpret_cast<const void*>(&k_backward<6>);
-    case 7: return reinterpret_cast<const void*>(&k_backward<7>);
-    case 8: return reinterpret_cast<const void*>(&k_backward<8>);
-    default: return nullptr;
-  }
+  return m == 1   ? reinterpret_cast<const void*>(&k_backward<1>)
+         : m == 2 ? reinterpret_cast<const void*>(&k_backward<2>)
+                  : nullptr;
 }
 
+// Head kernel of m rows and subtrees of G columns (G = 2 up to m = 4, 3 and 4
+// from m = 4 and 5 on).
 template <typename T, int M>
-const void* bwd_prefix_kernel_m() {
-  if constexpr (M >= 3) return reinterpret_cast<const void*>(&k_backward_prefix<T, M>);
-  else return nullptr;
+const void* bwd_heads_kernel_m(int G) {
+  if constexpr (M <= 4)
+    if (G == 2) return reinterpret_cast<const void*>(&k_backward_heads<T, M, 2>);
+  if constexpr (M >= 4)
+    if (G == 3) return reinterpret_cast<const void*>(&k_backward_heads<T, M, 3>);
+  if constexpr (M >= 5)
+    if (G == 4) return reinterpret_cast<const void*>(&k_backward_heads<T, M, 4>);
+  return nullptr;
 }
 
 template <typename T>
-const void* bwd_prefix_kernel(int m) {
+const void* bwd_heads_kernel(int m, int G) {
   switch (m) {
-    case 3: return bwd_prefix_kernel_m<T, 3>();
-    case 4: return bwd_prefix_kernel_m<T, 4>();
-    case 5: return bwd_prefix_kernel_m<T, 5>();
-    case 6: return bwd_prefix_kernel_m<T, 6>();
-    case 7: return bwd_prefix_kernel_m<T, 7>();
-    case 8: return bwd_prefix_kernel_m<T, 8>();
+    case 3: return bwd_heads_kernel_m<T, 3>(G);
+    case 4: return bwd_heads_kernel_m<T, 4>(G);
+    case 5: return bwd_heads_kernel_m<T, 5>(G);
+    case 6: return bwd_heads_kernel_m<T, 6>(G);
+    case 7: return bwd_heads_kernel_m<T, 7>(G);
+    case 8: return bwd_heads_kernel_m<T, 8>(G);
     default: return nullptr;
   }
 }
 
-// Work split of the prefix backward: prefixes grouped by their last column v
-// (k = n-1-v candidate columns), warp tasks of 32 lanes x a run of prefixes,
-// run lengths from a cost model (factorisation m P^2 + P^3, per candidate
-// column m + 4P and 2(m + P) gradient entries), `chunks` blocks per matrix.
-void bwd_prefix_plan(int batch, int m, int n, int sms, int* chunks, PrefixTable* tab) {
-  const int P = m - 2;
-  PrefixTable t;
-  std::memset(&t, 0, sizeof(t));
-  t.v_lo = P - 1;
-  t.v_hi = n - 3;
-  double cost[kMaxN] = {0}, total = 0.0;
-  for (int v = t.v_lo; v <= t.v_hi; ++v) {
-    const int k = n - 1 - v;
-    t.count[v] = binom_host(v, P - 1);
-    cost[v] = (double)m * P * P + (double)P * P * P + (double)k * (3.0 * m + 6.0 * P);
-    total += cost[v] * (double)t.count[v];
-  }
-  const long long want = (long long)(sms > 0 ? sms : 1) * 16;  // about 16 blocks per SM in all
-  long long ch = (want + batch - 1) / batch;
-  if (ch > 65535) ch = 65535;
-  if (ch < 1) ch = 1;
-  const double per_lane = total / ((double)ch * kBwdThreads) / 2.0;  // about two tasks per warp
-  unsigned long long start = 0;
-  for (int v = t.v_lo; v <= t.v_hi; ++v) {
-    double r = per_lane / cost[v];
-    unsigned long long run = r < 1.0 ? 1ull : (unsigned long long)r;
-    const unsigned long long maxrun = (t.count[v] + 31) / 32;
-    if (run > maxrun) run = maxrun > 0 ? maxrun : 1;
-    t.lanes[v] = 1;
-    t.run[v] = run;
-    t.task_start[v] = start;
-    start += (t.count[v] + 32 * run - 1) / (32 * run);
-  }
-  if (t.v_hi + 1 < kMaxN) t.task_start[t.v_hi + 1] = start;
-  t.total_tasks = start;
-  *chunks = (int)ch;
-  *tab = t;
-}
+struct BwdPlan {
+  int G = 0, chunks = 1;
+};
 
-size_t bwd_prefix_smem(int m, int n) {  // binary64 and pair elements are both 8 bytes
-  const int cs = ((m + 1) / 2) * 2;
-  size_t off = ((size_t)(n + 1) * (m + 1) * 8 + 15) / 16 * 16;
-  off += ((size_t)n * cs * 8 + 15) / 16 * 16;
-  off += ((size_t)m * n * 8 + 15) / 16 * 16;
-  off += (zbuf_bytes(n - m + 2, kBwdThreads, 2, 8) + 15) / 16 * 16;
-  const int ns = m - 2 > 2 ? m - 4 : 0;  // per-lane sums of the slow head columns
-  off += (size_t)ns * m * kBwdThreads * 8;
-  off += (size_t)(kBwdThreads / 32) * m * n * 8;  // the warps' gradient tiles
-  return off;
+// Subtree depth and blocks per matrix of the head kernel.  Estimate for every
+// available G, in binary64 warp instructions: a head's elimination, inverse and
+// prefix columns, per later column the three exterior products, the
+// contraction, Q and the m gradient entries with their warp sum.  An SM takes
+// one such instruction in 16 cycles from all its warps together, one warp of
+// its own every 64: the work spread over the SMs plus the longest task alone.
+// A block's four warps share a matrix; a matrix is split over several blocks
+// only as far as its tasks go, and until the batch gives every SM a few.
+BwdPlan bwd_plan(int batch, int m, int n, int sms) {
+  BwdPlan best;
+  double best_time = 0.0;
+  if (sms < 1) sms = 1;
+  for (int G = m <= 4 ? 2 : 3; G <= 4 && G < m; ++G) {
+    const int H = m - G;
+    const double ext = G * (double)(1 << (G - 1)) - G;
+    const double head = m * (double)H * H + 2.0 * H * H * H + H * (G * (double)H + (double)G * H + 3.0 * m) + 40.0;
+    const double col = 2.0 * G * H + 3.0 * ext + G * (double)(1 << (G - 1)) + 2.0 * G * H + G + 10.0;
+    double cols = 0.0, heads = 0.0;
+    for (int v = H - 1; v <= n - 1 - G; ++v) {
+      const double cnt = (double)binom_host(v, H - 1);
+      heads += cnt;
+      cols += cnt * (n - 1 - v);
+    }
+    const double tasks = std::ceil(heads / 32.0);
+    const double work = (double)batch * (tasks * head + std::max(cols / 32.0, cols / heads * tasks) * col);
+    const double longest = head + (n - H) * col;
+    const double time = 16.0 * work / sms + 64.0 * longest;
+    if (best.G == 0 || time < best_time) {
+      best.G = G;
+      best_time = time;
+      const long long by_work = ((long long)tasks + kBwdThreads / 32 - 1) / (kBwdThreads / 32);
+      const long long want = ((long long)sms * 8 + batch - 1) / batch;
+      best.chunks = (int)std::max(1ll, std::min(std::min(by_work, want), 65535ll));
+    }
+  }
+  return best;
 }
 
 int bwd_chunks(int batch, unsigned long long total) {
@@ -821,10 +975,7 @@ size_t radic_backward_workspace_bytes(int batch, int m, int n) {
   if (batch < 1 || m < 1 || m > kBwdMaxM || n < 1 || n > kMaxN) return 0;
   const unsigned long long total = (m <= n) ? binom_host(n, m) : 0ull;
   int chunks = bwd_chunks(batch, total);
-  if (m >= 3 && m <= n) {
-    PrefixTable tab;
-    bwd_prefix_plan(batch, m, n, device_sm_count(), &chunks, &tab);
-  }
+  if (m >= 3 && m <= n) chunks = bwd_plan(batch, m, n, device_sm_count()).chunks;
   return align_up((size_t)batch * chunks * m * n * sizeof(double), 256) + 256;
 }
 
@@ -861,21 +1012,24 @@ int radic_det_backward_mode(const double* A, int batch, int m, int n, int64_t ld
   a.total = binom_host(n, m);
   a.chunks = bwd_chunks(batch, a.total);
   a.slots = static_cast<double*>(workspace);
-  PrefixTable tab;
+  a.grad_out = grad_out;
+  a.grad = grad_A;
   const void* k;
   size_t smem;
-  if (m >= 3) {  // prefix-shared backward
-    bwd_prefix_plan(batch, m, n, device_sm_count(), &a.chunks, &tab);
-    k = (mode == RADIC_MODE_PAIR) ? bwd_prefix_kernel<ff>(m) : bwd_prefix_kernel<double>(m);
-    smem = bwd_prefix_smem(m, n);
+  if (m >= 3) {  // shared per head
+    const BwdPlan p = bwd_plan(batch, m, n, device_sm_count());
+    a.chunks = p.chunks;
+    k = (mode == RADIC_MODE_PAIR) ? bwd_heads_kernel<ff>(m, p.G) : bwd_heads_kernel<double>(m, p.G);
+    smem = BwdSmem<double>(nullptr, n, m, p.G, kBwdThreads / 32).bytes;
   } else {
     k = bwd_kernel(m);
     smem = bwd_smem(m, n);
   }
   if (!k || !allow_smem(k, smem)) return RADIC_EUNSUPPORTED;
-  void* params[] = {&a, &tab};
+  void* params[] = {&a};
   if (cudaLaunchKernel(k, dim3(a.chunks, batch), dim3(kBwdThreads), params, smem, s) != cudaSuccess)
     return RADIC_ECUDA;
+  if (m >= 3 && a.chunks == 1) return RADIC_OK;  // written by the kernel itself
   const long long total = (long long)batch * m * n;
   const unsigned blocks = (unsigned)std::min<long long>((total + 255) / 256, 65535);
   const double* slots = a.slots;
