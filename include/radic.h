@@ -323,7 +323,8 @@ typedef struct radic_batch_graph radic_batch_graph;
 /* Per-m tuning of the batched path (written by the autotuner; zero fields
  * mean "default").  kind[m]: RADIC_MAP_PREFIX or RADIC_MAP_THREAD (per-minor,
  * m <= 8).  task_cost[m]: target work per lane and task, in the plan's cost
- * units (default 30000; smaller = more, shorter tasks). */
+ * units (default 30000 for large batches, less for small ones; smaller =
+ * more, shorter tasks). */
 typedef struct radic_batch_tuning {
   int32_t kind[RADIC_MAX_M + 1];
   double task_cost[RADIC_MAX_M + 1];
@@ -377,7 +378,9 @@ int radic_batch_plan_destroy(radic_batch_plan* plan);
  * heads or C(n,m) ranks), then for head-shared tasks the segment of each
  * head's last prefix columns the task covers, vlo and vhi (last columns in
  * [vlo, vhi]); zeros otherwise.  Lane l of a task takes units
- * [r0 + l*run, min(r0 + (l+1)*run, lim)).  *n_tasks receives the total; rows
+ * [r0 + l*run, min(r0 + (l+1)*run, lim)); the last task of a binary64 prefix
+ * or head group, with fewer runs than lanes, may give two or more neighbouring
+ * lanes to each run.  *n_tasks receives the total; rows
  * past capacity are not written.  Errors as radic_batch_plan_create's
  * planning (RADIC_EINVAL, RADIC_EUNSUPPORTED). */
 #define RADIC_BATCH_TASK_FIELDS 10

@@ -33,6 +33,7 @@ SOURCES = [
     "radic_batched_k32.cu",
     "radic_batched_kpair.cu",
     "radic_batched_k64.cu",
+    "radic_batched_k64_hi.cu",
     "radic_backward.cu",
 ]
 

@@ -12,12 +12,13 @@
 
 namespace radic {
 
+namespace {
+constexpr BinomConst kBinomHost = make_binom_const();
+}
+
 unsigned long long binom_host(int n, int k) {
   if (k < 0 || k > n) return 0ull;
-  unsigned long long c[kMaxN + 1] = {1ull};
-  for (int v = 1; v <= n; ++v)
-    for (int j = (v < k ? v : k); j >= 1; --j) c[j] += c[j - 1];
-  return c[k];
+  return kBinomHost.v[n][k];
 }
 
 int device_sm_count() {
@@ -170,19 +171,25 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
     int lp = 1;
     if (d.lanes_per_prefix > 0) {
       lp = d.lanes_per_prefix;
-    } else if (D == 3) {
-      // Only depth 3 (its leaves grow like C(k, 3); splitting depth-2
-      // prefixes measured slower).  Target with binary32 elimination: 1.4
+    } else if (D == 3 || (pl.mode == kModeFp64 && m >= 4)) {
+      // Depth 3 (its leaves grow like C(k, 3)), and binary64 depth 2, whose
+      // small launches otherwise leave most SMs idle behind one lane's chain
+      // of binary64 operations (5 x 16: 5 blocks on 152 SMs).  In the other
+      // modes splitting depth-2 prefixes measured slower.  Target with binary32 elimination: 1.4
       // times the mean lane work when that is large, three times when the
       // launch is small and the repeated factorisations would dominate.
       // Binary64 and pair leaves keep their pipes busy, so there the balance
       // of the warps' shares matters more than the repeated work: the mean
       // itself.  (Measured on the shapes of prefix_auto_depth, warps drawing
       // tasks from the shared counter.)
-      const double mean = 4.0 * per_lane;
+      // Binary64 depth 2: the mean over one warp per scheduler, which is what
+      // keeps the binary64 pipe busy (over all resident lanes every group of a
+      // 6 x 24 matrix was split, and the repeated factorisations doubled its
+      // time).
+      const double mean = D == 2 ? total_cost / ((double)sms * 128.0) : 4.0 * per_lane;
       const double tf = (pl.mode == kModeMixed) ? (mean >= 1000.0 ? 1.4 : 3.0) : 1.0;
       const double target = tf * mean;
-      const double red = prefix_cost_shared(m, D, n - 1 - v), split = cost[v] - red;
+      const double red = (double)m * P * P, split = cost[v] - red;
       while (lp < 32 && red + split / lp > target) lp *= 2;
     }
     const unsigned long long groups = 32 / lp;  // lane groups per warp

@@ -85,38 +85,102 @@ double head_cost(int m, int D, int n, int v0, int v1) {
   return c;
 }
 
+// Work per lane and task, in the cost units above, when the tuning names none:
+// kTaskCost, or in binary64 about an eighth of a warp's share of the batch
+// (persistent kernels of eight warps on each of the GB300's 152 SMs) where that
+// is less, down to a floor below which staging the matrix again for every task
+// costs more than the balance gains: 1500, and 3000 where the matrices
+// themselves already make small or many tasks.  (Measured in binary64: 300
+// matrices, m = 2..9, n - m <= 16, 3.3 ms with kTaskCost for every batch, the
+// SMs busy 14 to 63% of the kernels' time, 1.5 ms now, 81 to 93% in the two
+// kernels with most work; 30 of 8 x (9..20) 1.28 ms, 0.23 with a floor of 3000,
+// 0.15 with 1500; 2000 with m = 2..6, n - m <= 20, 1.21 ms and 0.87 now.)
+constexpr double kTaskCost = 30000.0;
+double default_task_cost(double total_cost, int batch) {
+  constexpr double kWarps = 152.0 * 8.0;
+  const double share = total_cost / (kWarps * 32.0), per_matrix = total_cost / (batch * 32.0);
+  const double least = (batch > kWarps || per_matrix < 500.0) ? 3000.0 : 1500.0;
+  return std::min(kTaskCost, std::max(least, share / 8.0));
+}
+
 // Minors one lane works for one unit of a head-shared task at most (a single
 // prefix, up to C(n-m+D, D) minors, is never split): a head's whole subtree
 // holds up to C(n-m+1, D+1) minors, and the longest unit sets the kernel's
-// critical path.
-constexpr unsigned long long kSegmentMinors = 4096;
+// critical path.  Scales with the task cost.
+unsigned long long segment_minors(double task_cost) {
+  return (unsigned long long)(4096.0 * std::min(1.0, task_cost / kTaskCost));
+}
 
 // Splits the last columns v = u+1 .. n-1-D of the heads with last column u
-// into consecutive ranges of at most kSegmentMinors minors.
-std::vector<std::pair<int, int>> head_segments(int n, int D, int u) {
+// into consecutive ranges of at most `most` minors.
+std::vector<std::pair<int, int>> head_segments(int n, int D, int u, unsigned long long most) {
   std::vector<std::pair<int, int>> out;
   const int ve = n - 1 - D;
   int v = u + 1;
   while (v <= ve) {
     int v1 = v;
     unsigned long long sm = binom_host(n - 1 - v, D);
-    while (v1 + 1 <= ve && sm + binom_host(n - 2 - v1, D) <= kSegmentMinors) sm += binom_host(n - 1 - ++v1, D);
+    while (v1 + 1 <= ve && sm + binom_host(n - 2 - v1, D) <= most) sm += binom_host(n - 1 - ++v1, D);
     out.push_back({v, v1});
     v = v1 + 1;
   }
   return out;
 }
 
-int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* tun) {
-  const int m = pl.shape[2 * b], n = pl.shape[2 * b + 1];
-  std::vector<BatchTask>& out = (tier == kModeFp64) ? pl.t64 : pl.t32;
-  if (m > n) return RADIC_OK;
+// Task kind of a matrix: per minor or the prefix depth.
+int task_kind(int m, int n, int tier, const radic_batch_tuning* tun) {
   int kind = (m >= 3) ? prefix_auto_depth(m, n, true) : kKindMinor;
   if (tun && tun->kind[m] == RADIC_MAP_THREAD && m <= 8 && tier == kModeMixed) kind = kKindMinor;
   if (tun && tun->kind[m] == RADIC_MAP_PREFIX && m >= 3) kind = prefix_auto_depth(m, n, true);
   if (kind != kKindMinor && tun && (tun->prefix_depth[m] == 2 || (tun->prefix_depth[m] == 3 && m >= 4)))
     kind = tun->prefix_depth[m];
-  const double lane_cost = (tun && tun->task_cost[m] > 0.0) ? tun->task_cost[m] : 30000.0;
+  return kind;
+}
+
+// Estimated work of a matrix over all its units, in lane cost units.
+double matrix_cost(int m, int n, int kind) {
+  if (m > n) return 0.0;
+  if (kind == kKindMinor) return cost_minor(m) * (double)binom_host(n, m);
+  double c = 0.0;
+  for (int v = m - kind - 1; v <= n - 1 - kind; ++v)
+    c += (double)binom_host(v, m - kind - 1) * prefix_cost(m, kind, n - 1 - v);
+  return c;
+}
+
+// Lanes sharing each unit of a task that holds `units` runs (at most 32): a
+// task with fewer runs than lanes (the groups with the most candidate columns
+// hold the fewest prefixes) spreads each unit's columns and leaves over the
+// idle lanes, as far as the unit has work to share (`split`: its cost without
+// the part every lane repeats).  Binary64 only: the other tiers' sums of
+// |terms| are binary32 sums per prefix whose rounding would depend on it.
+int task_lanes(unsigned long long units, double split) {
+  int lp = 1;
+  while (units * lp * 2 <= 32 && split / lp > 200.0) lp *= 2;
+  return lp;
+}
+
+// Units per lane and task for a group of cnt units of cost c.  In binary64 the
+// group's tasks are evened out: with runs of the full cost the last task could
+// hold a fraction of a run per lane (256 x 6 x 28: 2.57 ms at a task cost of
+// 30000, 3.5 ms at 12000, before).
+unsigned long long task_run(unsigned long long cnt, double c, double lane_cost, int tier) {
+  unsigned long long run = (unsigned long long)std::max(1.0, std::floor(lane_cost / c));
+  run = std::max(1ull, std::min(run, (cnt + 31) / 32));
+  if (tier != kModeFp64) return run;
+  const unsigned long long tasks = (cnt + 32 * run - 1) / (32 * run);
+  return (cnt + 32 * tasks - 1) / (32 * tasks);
+}
+
+int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* tun, double auto_cost) {
+  const int m = pl.shape[2 * b], n = pl.shape[2 * b + 1];
+  std::vector<BatchTask>& out = (tier == kModeFp64) ? pl.t64 : pl.t32;
+  if (m > n) return RADIC_OK;
+  const int kind = task_kind(m, n, tier, tun);
+  // the pair tier's bounds follow the lanes' running totals, so its runs of
+  // prefixes do not depend on the batch
+  const double lane_cost = (tun && tun->task_cost[m] > 0.0) ? tun->task_cost[m]
+                           : tier == kModeFp64             ? auto_cost
+                                                           : kTaskCost;
   BatchTask t;
   std::memset(&t, 0, sizeof(t));
   t.offset = pl.offset[b];
@@ -125,6 +189,7 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
   t.n = n;
   t.kind = kind;
   t.tier = tier;
+  t.lp = 1;
   // Head sharing pays from heads of five columns on (measured on the batched
   // m = 5..10 sets: 25% faster at m = 10, depth 3; slower below four head
   // columns, where heads are few and their work uneven).
@@ -136,20 +201,21 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
     t.shared = 1;
     for (int u = H - 1; u <= n - 2 - D; ++u) {
       const unsigned long long cnt = binom_host(u, H - 1);
-      for (const auto& sg : head_segments(n, D, u)) {
+      for (const auto& sg : head_segments(n, D, u, segment_minors(lane_cost))) {
         const double c = head_cost(m, D, n, sg.first, sg.second);
-        unsigned long long run = (unsigned long long)std::max(1.0, std::floor(lane_cost / c));
-        run = std::min(run, (cnt + 31) / 32);
-        if (run < 1) run = 1;
+        const unsigned long long run = task_run(cnt, c, lane_cost, tier);
         t.vlo = sg.first;
         t.vhi = sg.second;
         t.per_unit = 0;
         for (int v = sg.first; v <= sg.second; ++v) t.per_unit += binom_host(n - 1 - v, D);
+        const double split = c - (double)m * H * H - (sg.second - sg.first + 1) * (m + 4.0 * (D + 1) * H);
         for (unsigned long long r0 = 0; r0 < cnt; r0 += 32 * run) {
           t.v = u;
           t.r0 = r0;
           t.run = run;
           t.lim = cnt;
+          t.lp = tier == kModeFp64 ? task_lanes((cnt - r0 + run - 1) / run, split) : 1;
+          t.cost = (double)run * c / t.lp;
           out.push_back(t);
         }
       }
@@ -159,15 +225,16 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
     for (int v = P - 1; v <= n - 1 - D; ++v) {
       const unsigned long long cnt = binom_host(v, P - 1);
       const double c = prefix_cost(m, D, n - 1 - v);
-      unsigned long long run = (unsigned long long)std::max(1.0, std::floor(lane_cost / c));
-      run = std::min(run, (cnt + 31) / 32);
-      if (run < 1) run = 1;
+      const unsigned long long run = task_run(cnt, c, lane_cost, tier);
       t.per_unit = binom_host(n - 1 - v, D);
+      const double split = c - (double)m * P * P;
       for (unsigned long long r0 = 0; r0 < cnt; r0 += 32 * run) {
         t.v = v;
         t.r0 = r0;
         t.run = run;
         t.lim = cnt;
+        t.lp = tier == kModeFp64 ? task_lanes((cnt - r0 + run - 1) / run, split) : 1;
+        t.cost = (double)run * c / t.lp;
         out.push_back(t);
       }
     }
@@ -177,6 +244,7 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
     run = std::min(run, (total + 31) / 32);
     if (run < 1) run = 1;
     t.per_unit = 1;
+    t.cost = (double)run * cost_minor(m);
     for (unsigned long long r0 = 0; r0 < total; r0 += 32 * run) {
       t.v = 0;
       t.r0 = r0;
@@ -186,12 +254,6 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
     }
   }
   return RADIC_OK;
-}
-
-double task_cost(const BatchTask& t) {
-  if (t.kind != kKindMinor && t.shared) return (double)t.run * head_cost(t.m, t.kind, t.n, t.vlo, t.vhi);
-  if (t.kind != kKindMinor) return (double)t.run * prefix_cost(t.m, t.kind, t.n - 1 - t.v);
-  return (double)t.run * cost_minor(t.m);
 }
 
 int persistent_blocks(const void* k, int slice_bytes, int sms) {
@@ -331,6 +393,7 @@ int plan_tasks(radic_batch_plan* pl, const int32_t* m, const int32_t* n, const i
   pl->shape.resize(2 * (size_t)batch);
   pl->offset.resize(batch);
   pl->tier.resize(batch);
+  double cost = 0.0;
   for (int b = 0; b < batch; ++b) {
     if (m[b] < 1 || n[b] < 1 || m[b] > kBatchMaxM || n[b] > kMaxN || offsets[b] < 0)
       return m[b] > kBatchMaxM && m[b] <= kMaxM ? RADIC_EUNSUPPORTED : RADIC_EINVAL;
@@ -362,18 +425,35 @@ int plan_tasks(radic_batch_plan* pl, const int32_t* m, const int32_t* n, const i
       pl->n_fp64_matrices++;
       pl->minors64 += c;
     }
-    make_tasks(*pl, b, tier, tuning);
+    cost += matrix_cost(m[b], n[b], task_kind(m[b], n[b], tier, tuning));
   }
+  const double auto_cost = default_task_cost(cost, batch);
+  for (int b = 0; b < batch; ++b) make_tasks(*pl, b, pl->tier[b], tuning, auto_cost);
   // per group (m, task path) and tier (binary32 before pairs), largest tasks
   // first (longest-processing-time order for each queue)
   auto gid = [](const BatchTask& t) { return group_of(t.m, path_of(t.kind, t.shared)); };
-  auto order = [&](const BatchTask& x, const BatchTask& y) {
-    if (gid(x) != gid(y)) return gid(x) < gid(y);
-    if (x.tier != y.tier) return x.tier == kModeMixed;
-    return task_cost(x) > task_cost(y);
+  struct Key {
+    int group, tier;
+    double cost;
+    size_t at;
   };
-  std::stable_sort(pl->t32.begin(), pl->t32.end(), order);
-  std::stable_sort(pl->t64.begin(), pl->t64.end(), order);
+  auto sort_tasks = [&](std::vector<BatchTask>& tasks) {
+    std::vector<Key> keys(tasks.size());
+    for (size_t i = 0; i < tasks.size(); ++i)
+      keys[i] = Key{gid(tasks[i]), tasks[i].tier == kModeMixed ? 0 : 1, tasks[i].cost, i};
+    std::sort(keys.begin(), keys.end(), [](const Key& x, const Key& y) {
+      if (x.group != y.group) return x.group < y.group;
+      if (x.tier != y.tier) return x.tier < y.tier;
+      if (x.cost != y.cost) return x.cost > y.cost;
+      return x.at < y.at;
+    });
+    std::vector<BatchTask> sorted;
+    sorted.reserve(tasks.size());
+    for (const Key& k : keys) sorted.push_back(tasks[k.at]);
+    tasks.swap(sorted);
+  };
+  sort_tasks(pl->t32);
+  sort_tasks(pl->t64);
   for (int g = 0; g <= kGroups; ++g) {
     pl->g32[g] = (int)(std::lower_bound(pl->t32.begin(), pl->t32.end(), g,
                                         [&](const BatchTask& t, int gg) { return gid(t) < gg; }) -
@@ -410,13 +490,16 @@ int radic_batch_plan_create(const int32_t* m, const int32_t* n, const int64_t* o
     }
   }
   // per-matrix task lists in task order (fixed summation order)
-  std::vector<std::vector<int>> per(batch);
-  for (size_t i = 0; i < pl->t32.size(); ++i) per[pl->t32[i].b].push_back((int)i);
-  for (size_t i = 0; i < pl->t64.size(); ++i) per[pl->t64[i].b].push_back((int)(pl->t32.size() + i));
   pl->csr_ptr.assign(batch + 1, 0);
-  for (int b = 0; b < batch; ++b) {
-    pl->csr_ptr[b + 1] = pl->csr_ptr[b] + (int)per[b].size();
-    for (int id : per[b]) pl->csr_idx.push_back(id);
+  for (const auto* list : {&pl->t32, &pl->t64})
+    for (const BatchTask& t : *list) ++pl->csr_ptr[t.b + 1];
+  for (int b = 0; b < batch; ++b) pl->csr_ptr[b + 1] += pl->csr_ptr[b];
+  pl->csr_idx.resize(pl->t32.size() + pl->t64.size());
+  {
+    std::vector<int> at(pl->csr_ptr.begin(), pl->csr_ptr.end() - 1);
+    int id = 0;
+    for (const auto* list : {&pl->t32, &pl->t64})
+      for (const BatchTask& t : *list) pl->csr_idx[at[t.b]++] = id++;
   }
   if (pl->csr_idx.empty()) pl->csr_idx.push_back(0);
   // per-warp shared-memory slices of each m's kernels: binomial table and
@@ -482,12 +565,12 @@ int radic_batch_plan_create(const int32_t* m, const int32_t* n, const int64_t* o
       for (int q = 0; q < 2; ++q) {
         if (ranges[q][1] <= ranges[q][0]) continue;
         double c = 0.0;
-        for (int i = ranges[q][0]; i < ranges[q][1]; ++i) c += task_cost(pl->t32[i]);
+        for (int i = ranges[q][0]; i < ranges[q][1]; ++i) c += pl->t32[i].cost;
         low.push_back({c, {q, g}});
       }
       if (pl->g64[g + 1] > pl->g64[g] || pl->g32[g + 1] > pl->g32[g]) {
         double c = 0.0;
-        for (int i = pl->g64[g]; i < pl->g64[g + 1]; ++i) c += task_cost(pl->t64[i]);
+        for (int i = pl->g64[g]; i < pl->g64[g + 1]; ++i) c += pl->t64[i].cost;
         hi.push_back({c, g});
       }
     }

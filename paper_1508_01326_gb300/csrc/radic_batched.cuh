@@ -52,9 +52,11 @@ struct BatchTask {
   int b, m, n, v;           // matrix, shape, prefix group
   int kind, tier;           // kKindMinor or the prefix depth; kModeMixed, kModePair or kModeFp64
   int shared;               // prefix kind: units are heads (first m-D-1 columns, v = their last column)
+  int lp;                   // lanes sharing each unit (prefix kinds, binary64; 1 otherwise)
   int vlo, vhi;             // head sharing: last prefix columns in [max(v+1, vlo), vhi] (a segment
                             // of each head's subtree)
   unsigned long long per_unit;  // minors under one unit (prefix, group segment or rank)
+  double cost;              // estimated lane work (host planning)
 };
 
 struct BatchHeader {
@@ -204,6 +206,8 @@ __device__ bool run_prefix(const BatchArgs& a, const BatchTask& t, const WarpSli
   constexpr int CS = ColStride<T, M>::value;
   constexpr int P = M - D;
   constexpr int H = P > 1 ? P - 1 : 1;
+  constexpr bool kSeq = std::is_same<T, double>::value;
+  const int lp = kSeq ? t.lp : 1, sub = kSeq ? (threadIdx.x & (t.lp - 1)) : 0;
   const int lane = threadIdx.x & 31;
   const T thr = static_cast<T>(a.growth);
   bool flagged = false;
@@ -218,7 +222,8 @@ __device__ bool run_prefix(const BatchArgs& a, const BatchTask& t, const WarpSli
     for (int j = 0; j < P - 1; ++j) c[j] = head[j];
     c[P - 1] = t.v;
     const bool f =
-        prefix_one<T, M, D, CS, false, kFlag>(w.As, w.binom, t.n, t.v, c, zb, thr, act, 0, 1, acc.p, ts, uin, w.As64);
+        prefix_one<T, M, D, CS, false, kFlag, kSeq>(w.As, w.binom, t.n, t.v, c, zb, thr, act, sub, lp, acc.p, ts, uin,
+                                                    w.As64);
     if (kFlag && act && f) flagged = true;
     acc.p.end_prefix();
     if constexpr (P > 1) {
@@ -241,6 +246,8 @@ __device__ bool run_prefix_heads(const BatchArgs& a, const BatchTask& t, const W
   constexpr int CS = ColStride<T, M>::value;
   constexpr int P = M - D, H = P - 1;
   static_assert(H >= 2, "head sharing needs a head of two or more columns");
+  constexpr bool kSeq = std::is_same<T, double>::value;
+  const int lp = kSeq ? t.lp : 1, sub = kSeq ? (threadIdx.x & (t.lp - 1)) : 0;
   const int lane = threadIdx.x & 31;
   const int u = t.v;
   const T thr = static_cast<T>(a.growth);
@@ -292,8 +299,8 @@ __device__ bool run_prefix_heads(const BatchArgs& a, const BatchTask& t, const W
                                      idx, prod, gmax, neg, pe.rel_alpha, pe.bad);
       }
       pe.kappa = 0.0f;
-      const bool f = prefix_leaves<T, M, D, CS, false, kFlag>(w.As, w.binom, t.n, v, c, W, idx, prod, gmax, neg, zb,
-                                                              thr, act, 0, 1, acc.p, ts, pe, rW, uin);
+      const bool f = prefix_leaves<T, M, D, CS, false, kFlag, kSeq>(w.As, w.binom, t.n, v, c, W, idx, prod, gmax, neg,
+                                                                    zb, thr, act, sub, lp, acc.p, ts, pe, rW, uin);
       if (kFlag && act && f) flagged = true;
       acc.p.end_prefix();
     }
@@ -310,7 +317,7 @@ __device__ bool run_task(const BatchArgs& a, const BatchTask& t, const WarpSlice
   const int lane = threadIdx.x & 31;
   const T thr = static_cast<T>(a.growth);
   bool flagged = false;
-  const unsigned long long first = t.r0 + (unsigned long long)lane * t.run;
+  const unsigned long long first = t.r0 + (unsigned long long)(lane / t.lp) * t.run;
   const unsigned long long last = min(first + t.run, t.lim);
   if constexpr (PATH == 3) {
     if constexpr (M >= 5) flagged = run_prefix_heads<T, M, 2, kFlag>(a, t, w, acc, first, last, uin);
@@ -396,7 +403,7 @@ __device__ void do_task(const BatchArgs& a, const BatchTask& t, unsigned char* s
       // count: minors of a binary32 or pair task recomputed here in binary64
       long long redone = 0;
       if (!kFlag && t.tier != kModeFp64) {
-        const unsigned long long units = min(32ull * t.run, t.lim - t.r0);
+        const unsigned long long units = min(32ull / t.lp * t.run, t.lim - t.r0);
         redone = (long long)(units * t.per_unit);
       }
       a.slots[slot_id] = FpPartial{d.hi, d.lo, ab, redone, bnd, 0.0};
@@ -409,8 +416,17 @@ __device__ void do_task(const BatchArgs& a, const BatchTask& t, unsigned char* s
 // Binary64 tier: queue over this group's binary64 tasks, then over its
 // binary32 and pair tasks that were flagged or rerouted (their slots are
 // overwritten with binary64 sums).
+// Register caps of the binary64 kernels by the blocks their shared memory
+// lets in: two from eight rows on, three below, four up to five rows.  Left to
+// itself the compiler settled for 168 registers and 4 KB of spills per thread
+// at ten rows, and for 128 and spills at six.  0: the compiler decides.
+template <typename T, int M>
+__host__ __device__ constexpr int batch_min_blocks() {
+  return !std::is_same<T, double>::value ? 0 : M >= 8 ? 2 : M >= 6 ? 3 : 4;
+}
+
 template <typename T, bool kMixedTier, int M, int PATH>
-__global__ void __launch_bounds__(kBatchThreads) k_batch(BatchArgs a) {
+__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<T, M>()) k_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char* slice = smem_raw + (size_t)warp * a.slice_bytes;
@@ -542,22 +558,15 @@ const void* batch_kernel_m(int path) {
   }
 }
 
-// Kernel of one tier for group (m, path), or nullptr where the path does not
-// apply (path_valid).
-template <typename T, bool kMixed>
+// Kernel of one tier for group (m, path) with LO <= m <= HI, or nullptr where
+// the path does not apply (path_valid).
+template <typename T, bool kMixed, int LO = 1, int HI = kBatchMaxM>
 const void* batch_kernel(int m, int path) {
-  switch (m) {
-    case 1: return batch_kernel_m<T, kMixed, 1>(path);
-    case 2: return batch_kernel_m<T, kMixed, 2>(path);
-    case 3: return batch_kernel_m<T, kMixed, 3>(path);
-    case 4: return batch_kernel_m<T, kMixed, 4>(path);
-    case 5: return batch_kernel_m<T, kMixed, 5>(path);
-    case 6: return batch_kernel_m<T, kMixed, 6>(path);
-    case 7: return batch_kernel_m<T, kMixed, 7>(path);
-    case 8: return batch_kernel_m<T, kMixed, 8>(path);
-    case 9: return batch_kernel_m<T, kMixed, 9>(path);
-    case 10: return batch_kernel_m<T, kMixed, 10>(path);
-    default: return nullptr;
+  if constexpr (LO <= HI) {
+    if (m == LO) return batch_kernel_m<T, kMixed, LO>(path);
+    return batch_kernel<T, kMixed, LO + 1, HI>(m, path);
+  } else {
+    return nullptr;
   }
 }
 

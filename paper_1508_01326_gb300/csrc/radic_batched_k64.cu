@@ -1,8 +1,8 @@
-// Persistent kernels of the batched path, binary64 tier (and the binary64 redo of flagged tasks), one per m and task path.
+// Binary64 kernels of the batched path, up to 8 rows.
 #include "radic_batched.cuh"
 
 namespace radic {
-
-const void* batch_kernel_f64(int m, int path) { return batch_kernel<double, false>(m, path); }
-
+const void* batch_kernel_f64(int m, int path) {
+  return m <= 8 ? batch_kernel<double, false, 1, 8>(m, path) : batch_kernel_f64_hi(m, path);
+}
 }  // namespace radic

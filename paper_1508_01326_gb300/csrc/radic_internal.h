@@ -184,6 +184,7 @@ size_t smem_modp(const SinglePlan& p, int use);
 const void* batch_kernel_f32(int m, int path);
 const void* batch_kernel_pair(int m, int path);
 const void* batch_kernel_f64(int m, int path);
+const void* batch_kernel_f64_hi(int m, int path);  // m >= 9
 
 // Prefix kernels of the EXACT mode (arguments: SingleArgs, PrefixTable), or
 // nullptr: per-minor terms for (m, depth); subtree sums for heads of m - G
@@ -209,14 +210,6 @@ inline double prefix_cost(int m, int D, int k) {
   double c = (double)m * P * P + (double)k * (m + 2.0 * D * P) + 6.0 * (double)binom_host(k, D);
   if (D == 3) c += 8.0 * (double)binom_host(k, 2);
   return c;
-}
-
-// The part of prefix_cost that every lane sharing one prefix repeats: the
-// factorisation (depth 3 lanes split the k column reductions as well as the
-// leaves; depth 2 does not split prefixes).
-inline double prefix_cost_shared(int m, int D, int k) {
-  const int P = m - D;
-  return (double)m * P * P + (D == 3 ? 0.0 : (double)k * (m + 2.0 * D * P));
 }
 
 // Default prefix depth for an m x n matrix.  Depth 3 divides the number of

@@ -39,6 +39,12 @@ struct ZBuf<T, 2> {
   V* p;
   int stride;
   __device__ ZBuf(void* base, int lane, int stride_, int /*kcap*/) : p(static_cast<V*>(base) + lane), stride(stride_) {}
+  // the buffer of the lane `d` positions away
+  __device__ __forceinline__ ZBuf shifted(int d) const {
+    ZBuf b = *this;
+    b.p += d;
+    return b;
+  }
   __device__ __forceinline__ void get(int q, T (&y)[2]) const {
     const V v = p[q * stride];
     y[0] = v.x;
@@ -57,6 +63,11 @@ struct ZBuf<ff, 2> {  // (x.hi, x.lo, y.hi, y.lo) in one 16-byte vector
   int stride;
   __device__ ZBuf(void* base, int lane, int stride_, int /*kcap*/)
       : p(static_cast<float4*>(base) + lane), stride(stride_) {}
+  __device__ __forceinline__ ZBuf shifted(int d) const {
+    ZBuf b = *this;
+    b.p += d;
+    return b;
+  }
   __device__ __forceinline__ void get(int q, ff (&y)[2]) const {
     const float4 v = p[q * stride];
     y[0] = ff(v.x, v.y);
@@ -499,6 +510,12 @@ struct LeafBound {
   // |z_d - z^_d| <= sum_j rW_dj |x_j| + (P u + u_in)(|x_Bd| + sum_j |W_dj| |x_j|)
   //              = cround |x_Bd| + sum_j cW_dj |x_j|
   __device__ __forceinline__ void column(const T (&z)[D], const R (&ax)[P + D]) {
+    R n, r;
+    column_radius(z, ax, n, r);
+    if constexpr (kOn) poly.add(n, r);
+  }
+  // the column's ||z^|| and radius alone
+  __device__ __forceinline__ void column_radius(const T (&z)[D], const R (&ax)[P + D], R& n, R& r) {
     if constexpr (kExact) {
       R n2 = R(0), r2 = R(0);
 #pragma unroll
@@ -510,7 +527,8 @@ struct LeafBound {
         for (int j = 0; j < P; ++j) rz = fmaf(cW[d][j], ax[j], rz);
         r2 += rz * rz;
       }
-      poly.add(sqrt(n2) * R(1.0000005), sqrt(r2) * R(1.000002));
+      n = sqrt(n2) * R(1.0000005);
+      r = sqrt(r2) * R(1.000002);
     } else if constexpr (kOn) {
       R n2 = R(0), x2 = R(0);
 #pragma unroll
@@ -520,7 +538,8 @@ struct LeafBound {
       }
 #pragma unroll
       for (int s = 0; s < P + D; ++s) x2 += ax[s] * ax[s];
-      poly.add(sqrt(n2) * R(1.0000005), kappa * sqrt(x2) * R(1.000002));
+      n = sqrt(n2) * R(1.0000005);
+      r = kappa * sqrt(x2) * R(1.000002);
     }
   }
   __device__ __forceinline__ void term_abs(const T& babs) {
@@ -530,10 +549,12 @@ struct LeafBound {
 
 // Schur complement of candidate column `col`, with the sign of its index
 // parity and (first entry) the prefix scale alpha folded in; updates zmax.
+// With nr (kSeq groups, prefix_leaves) the column's norm and radius go there
+// instead of into the bound's sums.
 template <typename T, int M, int D, int CS, bool kB>
 __device__ __forceinline__ void leaf_column(const T* __restrict__ As, int col, const T (&W)[D][M - D],
                                             const int (&idx)[M], T alpha, T (&z)[D], T& zmax,
-                                            LeafBound<T, D, M - D, kB>& lb) {
+                                            LeafBound<T, D, M - D, kB>& lb, float* nr = nullptr) {
   constexpr int P = M - D;
   const T* cp = As + col * CS;
   T x[M];
@@ -555,7 +576,8 @@ __device__ __forceinline__ void leaf_column(const T* __restrict__ As, int col, c
     Rad<T> ax[M];
 #pragma unroll
     for (int s = 0; s < M; ++s) ax[s] = mag(x[s]);
-    lb.column(z, ax);
+    if (nr) lb.column_radius(z, ax, nr[0], nr[1]);
+    else lb.column(z, ax);
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -563,6 +585,12 @@ __device__ __forceinline__ void leaf_column(const T* __restrict__ As, int col, c
     if (col & 1) z[d] = -z[d];
   }
   z[0] *= alpha;
+}
+
+// Sum over the aligned group of lp lanes (lp a power of two).
+__device__ __forceinline__ double group_sum(double x, int lp) {
+  for (int off = 1; off < lp; off <<= 1) x += __shfl_xor_sync(kFull, x, off);
+  return x;
 }
 
 // Leaf phase of one prefix without per-leaf output: the k later columns are
@@ -578,8 +606,10 @@ __device__ __forceinline__ void leaf_column(const T* __restrict__ As, int col, c
 //
 // kCoop: the buffer already holds every column's z (written by the lanes
 // sharing the prefix, see prefix_leaves); the block's columns are read from
-// it instead of being reduced here.
-template <typename T, int M, int D, int CS, bool kCoop, bool kB>
+// it instead of being reduced here.  kSeq: the lanes' column sums are added
+// up over the group and the first lane takes them, column by column, as one
+// lane alone would.
+template <typename T, int M, int D, int CS, bool kCoop, bool kSeq, bool kB>
 __device__ __forceinline__ void prefix_leaves_blocked(const T* __restrict__ As, int v, int k, const T (&W)[D][M - D],
                                                       const int (&idx)[M], T alpha, const ZBuf<T, D>& zb, bool act,
                                                       int sub, int lp, PrefixAcc<T>& acc, T& zmax,
@@ -684,7 +714,11 @@ __device__ __forceinline__ void prefix_leaves_blocked(const T* __restrict__ As, 
       bsum += cs[b];
       babs += ca[b];
     }
-    if (act) {
+    if constexpr (kSeq) {
+      bsum = group_sum(bsum, lp);
+      babs = group_sum(babs, lp);
+    }
+    if (act && (!kSeq || sub == 0)) {
       acc.add_column(bsum, babs);
       lb.term_abs(babs);
     }
@@ -810,7 +844,12 @@ __device__ __noinline__ void prefix_minors_f64(const double* __restrict__ As, co
   }
 }
 
-template <typename T, int M, int D, int CS, bool kTerms, bool kRedo = true>
+// kSeq (binary64): lanes that share a prefix reproduce the error bound of one
+// lane working it alone bit for bit, whatever their number: the columns'
+// (norm, radius) pairs and the column sums of |terms| enter its sums one
+// column after the other (bounds are binary32 sums, whose rounding otherwise
+// depends on how many lanes share the prefix).
+template <typename T, int M, int D, int CS, bool kTerms, bool kRedo = true, bool kSeq = false>
 __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const uint64_t* binom, int n, int v,
                                               const int (&c)[M - D], const T (&W)[D][M - D], const int (&idx)[M],
                                               T prod, T gmax, bool neg, const ZBuf<T, D>& zb, T thr, bool act,
@@ -857,7 +896,44 @@ __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const ui
     prefix_leaves_terms<T, M, D, CS>(As, binom, n, v, k, W, idx, alpha, rank_prefix, zb, act, sub, lp, acc, zmax,
                                      ts, nan_out);
   } else {
-    if constexpr (D == 3) {
+    if constexpr (kSeq) {
+      // Two phases as below; each column's (norm, radius) goes to the buffer
+      // slot of the lane after the group's first (8 bytes per column, free
+      // when lp > 1), from which every lane takes all of them in order.
+      static_assert(sizeof(T) == 8, "one slot entry holds two binary32 numbers");
+      const ZBuf<T, D> zg = zb.shifted(-sub);
+      if (D == 2 && lp == 1) {
+        // one lane, depth 2: columns and leaves in one pass (two passes
+        // measured 11% slower on 256 x 6 x 28)
+        prefix_leaves_blocked<T, M, D, CS, false, false>(As, v, k, W, idx, alpha, zb, act, 0, 1, acc, zmax, lb);
+      } else if (lp == 1) {
+        for (int q = 0; q < k; ++q) {
+          T z[D];
+          leaf_column<T, M, D, CS>(As, v + 1 + q, W, idx, alpha, z, zmax, lb);
+          zg.put(q, z);
+        }
+      } else {
+        const ZBuf<T, D> ng = zg.shifted(1);
+        for (int q = sub; q < k; q += lp) {
+          T z[D];
+          float nr[2];
+          leaf_column<T, M, D, CS>(As, v + 1 + q, W, idx, alpha, z, zmax, lb, nr);
+          zg.put(q, z);
+          *reinterpret_cast<float2*>(&ng.p[q * ng.stride]) = make_float2(nr[0], nr[1]);
+        }
+        zmax = group_max(zmax, lp);
+        __syncwarp();
+        for (int q = 0; q < k; ++q) {
+          const float2 nr = *reinterpret_cast<const float2*>(&ng.p[q * ng.stride]);
+          lb.poly.add(nr.x, nr.y);
+        }
+      }
+      if (D == 3 || lp > 1) {
+        __syncwarp();
+        prefix_leaves_blocked<T, M, D, CS, true, true>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
+      }
+      __syncwarp();  // the buffer is rewritten by the group's next prefix
+    } else if constexpr (D == 3) {
       // Two phases.  The lp lanes sharing the prefix split its column
       // reductions: lane `sub` reduces the columns q = sub (mod lp) into the
       // group's buffer (the slots of the group's first lane); then each lane
@@ -874,17 +950,23 @@ __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const ui
       zmax = group_max(zmax, lp);
       group_combine(lb.poly, lp);
       __syncwarp();
-      prefix_leaves_blocked<T, M, D, CS, true>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
+      prefix_leaves_blocked<T, M, D, CS, true, false>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
       __syncwarp();  // the buffer is rewritten by the group's next prefix
     } else {
-      prefix_leaves_blocked<T, M, D, CS, false>(As, v, k, W, idx, alpha, zb, act, sub, lp, acc, zmax, lb);
+      prefix_leaves_blocked<T, M, D, CS, false, false>(As, v, k, W, idx, alpha, zb, act, sub, lp, acc, zmax, lb);
     }
   }
   bool bad = false;
   if constexpr (kB) {
     // this lane's share of the prefix's bound (radic_bound.cuh)
     R b = (pe.rel_alpha + B::u * leaf_sum_depth(D, k, leaf_block<T>())) * lb.pabs;
-    if (sub == 0)
+    if constexpr (kSeq) {
+      // rounding stated, so that it does not depend on what the compiler
+      // fuses where this is inlined: the same bits for every number of lanes
+      b = fma(mag(alpha) * (R(1) + pe.rel_alpha),
+              __fadd_rn(lb.poly.perturbation(), __fmul_rn(R(leaf_round_coef<D>()) * B::u, lb.poly.hadamard())), b);
+      if (sub != 0) b = R(0);
+    } else if (sub == 0)
       b += mag(alpha) * (R(1) + pe.rel_alpha) *
            (lb.poly.perturbation() + R(leaf_round_coef<D>()) * B::u * lb.poly.hadamard());
     if (act) acc.add_bound(b);
@@ -921,7 +1003,7 @@ __device__ __forceinline__ void prefix_to_pairs(const double (&Wd)[D][P], float 
 
 // Processes one prefix c[0..m-D-1] (last column v): factors it, then its
 // leaves (prefix_leaves).
-template <typename T, int M, int D, int CS, bool kTerms, bool kRedo = true>
+template <typename T, int M, int D, int CS, bool kTerms, bool kRedo = true, bool kSeq = false>
 __device__ __forceinline__ bool prefix_one(const T* __restrict__ As, const uint64_t* binom, int n, int v,
                                            const int (&c)[M - D], const ZBuf<T, D>& zb, T thr, bool act, int sub,
                                            int lp, PrefixAcc<T>& acc, const TermsSink& ts,
@@ -934,7 +1016,7 @@ __device__ __forceinline__ bool prefix_one(const T* __restrict__ As, const uint6
   bool neg;
   if constexpr (kTerms) {
     prefix_factor<T, M, D, CS>(As, c, W, idx, prod, gmax, neg);
-    return prefix_leaves<T, M, D, CS, kTerms, kRedo>(As, binom, n, v, c, W, idx, prod, gmax, neg, zb, thr, act, sub,
+    return prefix_leaves<T, M, D, CS, kTerms, kRedo, kSeq>(As, binom, n, v, c, W, idx, prod, gmax, neg, zb, thr, act, sub,
                                                      lp, acc, ts);
   } else {
     Rad<T> rW[D][P];
@@ -948,7 +1030,7 @@ __device__ __forceinline__ bool prefix_one(const T* __restrict__ As, const uint6
       prefix_factor_b<T, M, D, CS>(As, c, W, rW, idx, prod, gmax, neg, pe.rel_alpha, pe.bad, uin);
     }
     pe.kappa = 0.0f;
-    return prefix_leaves<T, M, D, CS, kTerms, kRedo>(As, binom, n, v, c, W, idx, prod, gmax, neg, zb, thr, act, sub,
+    return prefix_leaves<T, M, D, CS, kTerms, kRedo, kSeq>(As, binom, n, v, c, W, idx, prod, gmax, neg, zb, thr, act, sub,
                                                      lp, acc, ts, pe, rW, uin);
   }
 }
@@ -1243,6 +1325,9 @@ __global__ void __launch_bounds__(128, prefix_min_blocks<T>()) k_fp_prefix(Singl
   static_assert(M > D, "the prefix needs at least one column");
   constexpr int P = M - D;
   constexpr int CS = ColStride<T, M>::value;
+  // binary64 depth-2 prefixes shared by several lanes (small launches) keep
+  // the bound of one lane alone
+  constexpr bool kSeq = std::is_same<T, double>::value && D == 2 && !kTerms;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = a.n;
   FpSmem<T> sm(smem_raw, n, M, CS);
@@ -1300,8 +1385,8 @@ __global__ void __launch_bounds__(128, prefix_min_blocks<T>()) k_fp_prefix(Singl
 #pragma unroll
       for (int j = 0; j < P - 1; ++j) c[j] = head[j];
       c[P - 1] = v;
-      const bool flag = prefix_one<T, M, D, CS, kTerms, kMixed>(sm.As, sm.binom, n, v, c, zb, thr, act, sub, lp, acc,
-                                                                 ts, uin, sm.As64);
+      const bool flag = prefix_one<T, M, D, CS, kTerms, kMixed, kSeq>(sm.As, sm.binom, n, v, c, zb, thr, act, sub, lp,
+                                                                       acc, ts, uin, sm.As64);
       if constexpr (kMixed && !kTerms) {
         if (act && flag) acc.drop_prefix();  // its leaves are recomputed in binary64
         // every lane of the group drops its share; the first one records the prefix
