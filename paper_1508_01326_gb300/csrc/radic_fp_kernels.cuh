@@ -407,77 +407,141 @@ __device__ __forceinline__ T group_det(T (&x)[G], int m, int sub, int seg, T& gm
   return par ? -det : det;
 }
 
-// group_det with running error radii (binary32, one per entry of the
-// lane's row; radic_bound.cuh): the pivot row's radii travel with it by the
-// same shuffles.  bnd and bad are valid in every lane of the group.
-template <typename T, int G>
-__device__ __forceinline__ T group_det_b(T (&x)[G], int m, int sub, int seg, T& gmax, float& bnd, bool& bad,
-                                         float u_in = static_cast<float>(BoundTraits<T>::u_in)) {
-  constexpr float u = static_cast<float>(BoundTraits<T>::u);
-  constexpr float c_div = static_cast<float>(BoundTraits<T>::c_div);
-  float rx[G];
-#pragma unroll
-  for (int j = 0; j < G; ++j) rx[j] = u_in * mag(x[j]);
-  bool alive = sub < m;
-  T det = T(1);
-  int par = 0;
-  float rel = 0.0f, pr = 1.0f;  // pr = prod (|p_k| + r_k)
-  bool last_open = false;
-  bad = false;
-  gmax = T(0);
-  const unsigned segbits = (G == 32) ? kFull : ((1u << G) - 1u);
-#pragma unroll
-  for (int k = 0; k < G; ++k) {
-    if (k >= m) break;
-    uint32_t key = alive ? ((mag_key(x[k]) & ~31u) | (uint32_t)(G - 1 - sub)) : 0u;
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) key = max(key, __shfl_xor_sync(kFull, key, off));
-    const int p = G - 1 - (int)(key & 31u);
-    const T piv = __shfl_sync(kFull, x[k], p, G);
-    const float rp = __shfl_sync(kFull, rx[k], p, G);
-    const unsigned alive_bits = (__ballot_sync(kFull, alive) >> (seg * G)) & segbits;
-    par ^= __popc(alive_bits & ((1u << p) - 1u)) & 1;
-    if (sub == p) alive = false;
-    det *= piv;
-    gmax = fmax(gmax, fabs(piv));
-    const float ap = mag(piv);
-    pr *= ap + rp;
-    const float ipm = ap > 0.0f ? __frcp_ru(ap) : 0.0f;
-    const float ipd = ap > rp ? __frcp_ru(__fsub_rd(ap, rp)) : 0.0f;
-    if (k == m - 1) {
-      // the last pivot divides nothing: a singular minor is bounded by the
-      // product of the pivot enclosures instead
-      last_open = pivot_unbounded(ap, rp) || ap == 0.0f;
-    } else {
-      bad |= pivot_unbounded(ap, rp);
+// Partial-pivot LU of consecutive minors by a group of G lanes, column by
+// column (left-looking), with running error radii (binary32, one per entry;
+// radic_bound.cuh).  Consecutive minors of a run differ in their last columns
+// only, and elimination steps 0..k-1 of a column look at nothing but the
+// columns before it: the group keeps the multipliers of every step and resumes
+// at the first column that changed, about two columns per minor instead of m.
+// The operations on each entry and their order are those of eliminating every
+// minor from scratch, and so are the results.
+//
+// Lane `sub` holds row `sub`: its multiplier of every step (0 once the row has
+// been a pivot) with magnitude and radius, the pivot rows, and, as lane j, the
+// determinant so far, radii, flags and rows left after step j (kGrowth: the
+// largest pivot too).
+//
+// What bounds it: shuffles (two for the pivot row's entry, one for its radius
+// per step) and the binary64 pipe, one multiply-add per step and warp however
+// few lanes are rows.  12 x 20 (126 thousand minors): 751 us with every minor
+// eliminated on its own, 405 us now (the pipe 58% busy while the SMs are, which
+// is 76% of the time: later minors of dictionary order change more columns).
+template <typename T, int G, bool kGrowth>
+struct GroupLu {
+  T l[G];
+  float al[G], rl[G];
+  int p[G];
+  // lane j: state after step j
+  T det_s, gmax_s;
+  float rel_s, pr_s;
+  unsigned alive_s;  // rows left
+  int flags_s;       // bit 0 parity of the row permutation, bit 1 a pivot's enclosure reached zero
+
+  // Eliminates the minor whose columns c[first..m-1] are new; As: staged
+  // matrix (column stride m).  `first` is the same in every group of the warp.
+  // Returns det; bnd, bad and gmax are valid in every lane of the group.
+  __device__ __forceinline__ T run(const T* __restrict__ As, const int (&c)[G], int first, int m, int sub, T& gmax,
+                                   float& bnd, bool& bad, float u_in) {
+    constexpr float u = static_cast<float>(BoundTraits<T>::u);
+    constexpr float c_div = static_cast<float>(BoundTraits<T>::c_div);
+    const int prev = first > 0 ? first - 1 : 0;
+    T det = __shfl_sync(kFull, det_s, prev, G);
+    if constexpr (kGrowth) gmax = __shfl_sync(kFull, gmax_s, prev, G);
+    else gmax = T(0);
+    float rel = __shfl_sync(kFull, rel_s, prev, G), pr = __shfl_sync(kFull, pr_s, prev, G);
+    unsigned alive = __shfl_sync(kFull, alive_s, prev, G);
+    int flags = __shfl_sync(kFull, flags_s, prev, G);
+    if (first == 0) {
+      det = T(1);
+      gmax = T(0);
+      rel = 0.0f;
+      pr = 1.0f;  // prod (|p_k| + r_k)
+      alive = m == 32 ? kFull : (1u << m) - 1u;
+      flags = 0;
     }
-    if (!last_open) rel = fmaf(1.0f + rel, rp * ipm, rel);
-    T r;
-    if constexpr (sizeof(T) == 8) r = rcp_f64(piv);
-    else r = rcp_f32(piv);
-    const T l = alive ? x[k] * r : T(0);
-    const float al = mag(l);
-    const float rl = alive ? (rx[k] + al * rp) * ipd + c_div * u * al : 0.0f;
+    int cs = 0;  // lane j: column c_j
 #pragma unroll
-    for (int j = k + 1; j < G; ++j) {
-      if (j < m) {
-        const T uj = __shfl_sync(kFull, x[j], p, G);
-        const float ru = __shfl_sync(kFull, rx[j], p, G);
-        const float au = mag(uj), old = mag(x[j]);
-        x[j] = fma(-l, uj, x[j]);
-        rx[j] += al * ru + (au + ru) * rl + u * (al * au + old);
+    for (int j = 0; j < G; ++j) cs = sub == j ? c[j] : cs;
+    bool last_open = false;
+    // one copy of the column body for every j (a copy per column measured half
+    // of its time in instruction fetches)
+#pragma unroll 1
+    for (int j = first; j < m; ++j) {
+      const int col = __shfl_sync(kFull, cs, j, G);
+      T x = sub < m ? As[col * m + sub] : T(0);
+      float rx = u_in * mag(x);
+#pragma unroll
+      for (int k = 0; k < G - 1; ++k) {
+        if (k >= j) break;  // the same in every lane of the warp
+        const T uj = __shfl_sync(kFull, x, p[k], G);
+        const float ru = __shfl_sync(kFull, rx, p[k], G);
+        const float old = mag(x), au = __shfl_sync(kFull, old, p[k], G);  // |uj| as its own lane forms it
+        x = fma(-l[k], uj, x);
+        // rx += al ru + (au + ru) rl + u (al au + old)
+        rx += fmaf(u, fmaf(al[k], au, old), fmaf(al[k], ru, __fmul_rn(au + ru, rl[k])));
+      }
+      const bool up = (alive >> sub) & 1u;
+      uint32_t key = up ? ((mag_key(x) & ~31u) | (uint32_t)(G - 1 - sub)) : 0u;
+#pragma unroll
+      for (int off = G / 2; off > 0; off >>= 1) key = max(key, __shfl_xor_sync(kFull, key, off));
+      const int pk = G - 1 - (int)(key & 31u);
+      const T piv = __shfl_sync(kFull, x, pk, G);
+      const float rp = __shfl_sync(kFull, rx, pk, G);
+      flags ^= __popc(alive & ((1u << pk) - 1u)) & 1;
+      alive &= ~(1u << pk);
+      det *= piv;
+      if constexpr (kGrowth) gmax = fmax(gmax, fabs(piv));
+      const float ap = mag(piv);
+      pr *= ap + rp;
+      const float ipm = ap > 0.0f ? __frcp_ru(ap) : 0.0f;
+      const float ipd = ap > rp ? __frcp_ru(__fsub_rd(ap, rp)) : 0.0f;
+      if (j == m - 1) {
+        // the last pivot divides nothing: a singular minor is bounded by the
+        // product of the pivot enclosures instead
+        last_open = pivot_unbounded(ap, rp) || ap == 0.0f;
+        if (!last_open) rel = fmaf(1.0f + rel, rp * ipm, rel);
+        break;
+      }
+      if (pivot_unbounded(ap, rp)) flags |= 2;
+      rel = fmaf(1.0f + rel, rp * ipm, rel);
+      T r;
+      if constexpr (sizeof(T) == 8) r = rcp_f64(piv);
+      else r = rcp_f32(piv);
+      const bool still = up && sub != pk;
+      const T lj = still ? x * r : T(0);
+      const float aj = mag(lj);
+      const float rj = still ? fmaf(c_div * u, aj, __fmul_rn(fmaf(aj, rp, rx), ipd)) : 0.0f;
+#pragma unroll
+      for (int k = 0; k < G - 1; ++k) {
+        if (k == j) {
+          l[k] = lj;
+          al[k] = aj;
+          rl[k] = rj;
+          p[k] = pk;
+        }
+      }
+      if (sub == j) {
+        det_s = det;
+        if constexpr (kGrowth) gmax_s = gmax;
+        rel_s = rel;
+        pr_s = pr;
+        alive_s = alive;
+        flags_s = flags;
       }
     }
+    bad = (flags & 2) != 0;
+    rel = fmaf(1.0f + rel, static_cast<float>(m - 1) * u * 1.01f, rel);
+    bnd = last_open
+              ? (pr * (1.0f + static_cast<float>(m) * u) + static_cast<float>(m) * u * mag(det)) * 1.0000002f
+              : rel * mag(det) * 1.0000001f;
+    return (flags & 1) ? -det : det;
   }
-  rel = fmaf(1.0f + rel, static_cast<float>(m - 1) * u * 1.01f, rel);
-  bnd = last_open ? (pr * (1.0f + static_cast<float>(m) * u) + static_cast<float>(m) * u *
-                                                                      mag(det)) * 1.0000002f
-                  : rel * mag(det) * 1.0000001f;
-  return par ? -det : det;
-}
+};
 
+// Groups of 16: four blocks of 128 threads per SM (the plan's ranks per group
+// follow from it).  Groups of 32 hold twice the multipliers and would spill.
 template <typename T, int G, bool kMixed, bool kTerms>
-__global__ void __launch_bounds__(kMaxThreadsFp) k_fp_group(SingleArgs a) {
+__global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(SingleArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = a.n, m = a.m;
   FpSmem<T> sm(smem_raw, n, m, m);
@@ -492,13 +556,18 @@ __global__ void __launch_bounds__(kMaxThreadsFp) k_fp_group(SingleArgs a) {
 
   const int lane = threadIdx.x & 31, sub = lane & (G - 1), seg = lane / G;
   constexpr int kSegs = 32 / G;
-  const unsigned long long gwarp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  // a block's warps take tasks a grid apart: minors late in dictionary order
+  // change more columns each, and neighbouring tasks on one SM would make it
+  // the last to finish
+  const unsigned long long gwarp = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const unsigned long long nsegs = (unsigned long long)gridDim.x * blockDim.x / G;
   const unsigned long long L = a.ranks_per_task;
   const unsigned long long qbase = kTerms ? a.q0 : 0ull;
   const unsigned long long qlim = kTerms ? a.q0 + a.count : a.total;
   const T thr = static_cast<T>(a.growth);
 
+  GroupLu<T, G, kMixed> lu;  // unused by the terms
+  double pend = 0.0;  // binary64: this lane's pending minor
   Dd acc;
   double abs_sum = 0.0, bnd = 0.0;
   int fcnt = 0;
@@ -514,19 +583,20 @@ __global__ void __launch_bounds__(kMaxThreadsFp) k_fp_group(SingleArgs a) {
     unrank_dyn<G>(q0, n, m, sm.binom, m + 1, c);
     Ff run;
     float run_abs = 0.0f, run_bnd = 0.0f;
+    int first = 0;  // first column that changed since the previous minor
     for (unsigned long long it = 0; it < L; ++it) {
       const unsigned long long q = q0 + it;
       const bool act = tact && q < q1;
-      T x[G];
-#pragma unroll
-      for (int j = 0; j < G; ++j) x[j] = (j < m && sub < m) ? sm.As[c[j] * m + sub] : T(0);
       T gmax, det;
       float b = 0.0f;
       bool bad = false;
       if constexpr (kTerms) {
+        T x[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) x[j] = (j < m && sub < m) ? sm.As[c[j] * m + sub] : T(0);
         det = group_det<T, G>(x, m, sub, seg, gmax);
       } else {
-        det = group_det_b<T, G>(x, m, sub, seg, gmax, b, bad, uin);
+        det = lu.run(sm.As, c, first, m, sub, gmax, b, bad, uin);
         if (bad && !kMixed) {  // Hadamard's inequality alone
           float h = 1.0f;
 #pragma unroll
@@ -559,11 +629,15 @@ __global__ void __launch_bounds__(kMaxThreadsFp) k_fp_group(SingleArgs a) {
           fcnt += __popc(fm);
         }
       } else {
-        if (lead) {
-          acc.add(static_cast<double>(det));
-          abs_sum += fabs(static_cast<double>(det));
-          run_bnd += b;
+        // lane it mod G keeps the minor; the group's lanes add theirs together
+        // every G minors (one two-sum per warp instead of one per minor)
+        if (act && sub == (int)(it & (G - 1))) pend = static_cast<double>(det);
+        if ((it & (G - 1)) == G - 1 || it + 1 == L) {
+          acc.add(pend);
+          abs_sum += fabs(pend);
+          pend = 0.0;
         }
+        if (lead) run_bnd += b;
       }
       if constexpr (!kTerms) {
         if ((it & 255) == 255) {
@@ -578,7 +652,8 @@ __global__ void __launch_bounds__(kMaxThreadsFp) k_fp_group(SingleArgs a) {
           run_bnd = 0.0f;
         }
       }
-      if (q + 1 < q1) successor_dyn<G>(c, n, m);
+      const int changed = q + 1 < q1 ? successor_dyn<G>(c, n, m) : m - 1;
+      if constexpr (!kTerms) first = __reduce_min_sync(kFull, changed);  // over the warp's groups
     }
     if constexpr (!kTerms) {
       if constexpr (kMixed) {
