@@ -145,20 +145,35 @@ __device__ inline uint64_t mix64(uint64_t z) {  // SplitMix64 finaliser
   return z ^ (z >> 31);
 }
 
+// Floating-point rows: e_i, the exponent of the lowest set bit among row i's
+// nonzero entries, and the width w_i = top_i + 1 - e_i, top_i the exponent of
+// the highest set bit: the integer row M_i = 2^-e_i A_i has |entry| < 2^w_i, so
+// ||M_i|| < sqrt(n) 2^w_i.  A zero row has e_i = 0 and no bits (all its
+// minors are zero).  Integer rows: the squared norm in binary32.
+struct RowStats {
+  int lo[kMaxM], hi[kMaxM];  // floating point: lowest and highest set bit
+  float sq[kMaxM];           // integers
+  float bits[kMaxM + 1];     // bits of the row's norm bound; [m]: log2 C(n,m)
+  double bits64[kMaxM + 1];
+  int nonfinite, needed, esum;
+  __device__ __forceinline__ bool zero(int i) const { return hi[i] == -0x7fffffff; }
+  __device__ __forceinline__ int exponent(int i) const { return zero(i) ? 0 : lo[i]; }
+  __device__ __forceinline__ int width(int i) const { return zero(i) ? 0 : hi[i] + 1 - lo[i]; }
+};
+
 // Shared-memory layout: binom | K x (n x cs) residues (column-major, Montgomery
-// form) | 2 x (m x n) scratch rows | m x m triangular factors | row bounds |
-// scratch words for reductions | counts | Montgomery constants | row exponents.
+// form) | 2 x (m x n) scratch rows | m x m triangular factors | scratch words
+// for reductions | Montgomery constants | row statistics.
 __host__ __device__ inline size_t modp_smem_bytes(int n, int m, int cs, int threads) {
   size_t off = ((size_t)(n + 1) * (m + 1) * 8 + 15) / 16 * 16;
   off += (size_t)kMaxPrimes * n * cs * 4;
   off += (2 * (size_t)m * n * 4 + 15) / 16 * 16;
   off += ((size_t)m * m * 4 + 15) / 16 * 16;
-  off += (size_t)(m + 1) * 12;
   off += (size_t)(threads / 32) * kMaxPrimes * 4;
   off = (off + 15) / 16 * 16;
-  off += 64 + kMaxPrimes * sizeof(Mont);
-  off += (size_t)kMaxM * 8;  // row exponents and widths of floating-point inputs
-  return (off + 15) / 16 * 16;
+  off += kMaxPrimes * sizeof(Mont);
+  off = (off + 15) / 16 * 16;
+  return off + (sizeof(RowStats) + 15) / 16 * 16;
 }
 
 struct ModpSmem {
@@ -166,12 +181,9 @@ struct ModpSmem {
   uint32_t* As;  // prime k at As + k * n * cs
   uint32_t* rows;
   uint32_t* tri;
-  double* row_bits;
-  float* bits32;
   uint32_t* scratch;
-  int* misc;  // [0] primes the bound needs, [1] total row exponent, [2] non-finite flag
   Mont* mont;
-  int* row_e;  // floating-point inputs: row i times 2^-row_e[i] is integer, of width row_e[m + i]
+  RowStats* stats;
   __device__ ModpSmem(unsigned char* base, int n, int m, int cs, int threads) {
     size_t off = ((size_t)(n + 1) * (m + 1) * 8 + 15) / 16 * 16;
     binom = reinterpret_cast<uint64_t*>(base);
@@ -181,18 +193,13 @@ struct ModpSmem {
     off += (2 * (size_t)m * n * 4 + 15) / 16 * 16;
     tri = reinterpret_cast<uint32_t*>(base + off);
     off += ((size_t)m * m * 4 + 15) / 16 * 16;
-    row_bits = reinterpret_cast<double*>(base + off);
-    off += (size_t)(m + 1) * 8;
-    bits32 = reinterpret_cast<float*>(base + off);
-    off += (size_t)(m + 1) * 4;
     scratch = reinterpret_cast<uint32_t*>(base + off);
     off += (size_t)(threads / 32) * kMaxPrimes * 4;
     off = (off + 15) / 16 * 16;
-    misc = reinterpret_cast<int*>(base + off);
-    off += 64;
     mont = reinterpret_cast<Mont*>(base + off);
     off += kMaxPrimes * sizeof(Mont);
-    row_e = reinterpret_cast<int*>(base + off);
+    off = (off + 15) / 16 * 16;
+    stats = reinterpret_cast<RowStats*>(base + off);
   }
 };
 
@@ -259,120 +266,152 @@ __device__ __forceinline__ uint32_t int_residue(long long v, uint32_t p) {
   return static_cast<uint32_t>(v >= (long long)p ? v - p : v);
 }
 
-// Row exponents e_i (row_e[i]) and, per row, the width w_i (row_e[m + i]) of
-// a bound on the Euclidean norm of the integer row: |entry| < 2^w_i with
-// w_i = top_i + 1 - e_i, top_i the exponent of the highest set bit, so
-// ||M_i|| < sqrt(n) 2^w_i.  A zero row has e_i = 0 and width 0, for no bits
-// (all its minors are zero).  Sets *nonfinite (shared) when an entry is
-// infinite or NaN.
-__device__ inline void fp_row_scales(const void* A, int dtype, int m, int n, long long lda, int* row_e,
-                                     int* nonfinite) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = warp; i < m; i += nw) {
-    int lo = 0x7fffffff, hi = -0x7fffffff;
-    bool bad = false;
-    for (int j = lane; j < n; j += 32) {
-      const FpBits f = fp_bits(load_fp(A, dtype, (long long)i * lda + j));
-      if (!f.finite) {
-        bad = true;
-      } else if (f.mant) {
-        lo = min(lo, f.t + __ffsll(static_cast<long long>(f.mant)) - 1);
-        hi = max(hi, f.t + 63 - __clzll(static_cast<long long>(f.mant)));
-      }
+// ---------------------------------------------------------------------------
+// Staging.  One pass loads the matrix, each thread keeping its first kKeep
+// entries in registers, and forms the row statistics in shared memory; the
+// residues, U A and L (U A) are one pass of the block each.  (Row by row, a
+// warp per row and a binary64 sum and logarithm per row, this took 2.5 us of
+// a 3 x 12 call and 6 us of 10 x 24.)
+// ---------------------------------------------------------------------------
+constexpr int kKeepModp = 4;
+struct KeptEntries {
+  double f[kKeepModp];
+  int v[kKeepModp];
+};
+
+// Statistics of every row, the first kKeepModp entries of every thread kept.
+// Ends with a barrier.
+__device__ inline void row_stats(const SingleArgs& a, int m, RowStats& st, KeptEntries& keep) {
+  const int n = a.n, mn = m * n;
+  const bool fp = is_fp_dtype(a.dtype);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    st.lo[i] = 0x7fffffff;
+    st.hi[i] = -0x7fffffff;
+  }
+  if (threadIdx.x == 0) st.nonfinite = 0;
+  __syncthreads();
+  auto bits_of = [&](int i, double f) {
+    const FpBits x = fp_bits(f);
+    if (!x.finite) {
+      st.nonfinite = 1;
+    } else if (x.mant) {
+      atomicMin(&st.lo[i], x.t + __ffsll(static_cast<long long>(x.mant)) - 1);
+      atomicMax(&st.hi[i], x.t + 63 - __clzll(static_cast<long long>(x.mant)));
     }
-    lo = __reduce_min_sync(kFull, lo);
-    hi = __reduce_max_sync(kFull, hi);
-    bad = __any_sync(kFull, bad);
-    if (lane == 0) {
-      const bool zero = hi == -0x7fffffff;
-      row_e[i] = zero ? 0 : lo;
-      row_e[m + i] = zero ? 0 : hi + 1 - lo;
-      if (bad) *nonfinite = 1;
+  };
+#pragma unroll
+  for (int k = 0; k < kKeepModp; ++k) {
+    const int idx = threadIdx.x + k * blockDim.x;
+    if (idx < mn) {
+      const int i = idx / n;
+      const long long at = (long long)i * a.lda + (idx - i * n);
+      if (fp) keep.f[k] = load_fp(a.A, a.dtype, at);
+      else keep.v[k] = static_cast<int>(load_int(a.A, a.dtype, at));
     }
   }
-}
-
-// Bits of a bound on |det_R(A)| from the rows: C(n,m) prod_i ||row_i||_2
-// (Hadamard's inequality for every minor).  Integer rows by their norms, one
-// warp per row; floating-point rows by the widths of fp_row_scales.  Type F:
-// double as the count of primes is defined, float for the estimate below.
-// bits: m + 1 words of shared scratch, left with the rows' bits and
-// log2 C(n,m); ends with a barrier.
-template <typename F>
-__device__ inline void hadamard_bits(const SingleArgs& a, int m, double count, const int* row_e, F* bits) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (is_fp_dtype(a.dtype)) {
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      const int w = row_e[m + i];
-      bits[i] = w == 0 ? F(0) : static_cast<F>(w) + F(0.5) * log2(static_cast<F>(a.n));
+  if (fp) {
+#pragma unroll
+    for (int k = 0; k < kKeepModp; ++k) {
+      const int idx = threadIdx.x + k * blockDim.x;
+      if (idx < mn) bits_of(idx / n, keep.f[k]);
+    }
+    for (int idx = threadIdx.x + kKeepModp * blockDim.x; idx < mn; idx += blockDim.x) {
+      const int i = idx / n;
+      bits_of(i, load_fp(a.A, a.dtype, (long long)i * a.lda + (idx - i * n)));
     }
   } else {
-    for (int i = warp; i < m; i += nw) {
-      F s = F(0);
-      for (int j = lane; j < a.n; j += 32) {
-        const F v = static_cast<F>(load_int(a.A, a.dtype, (long long)i * a.lda + j));
-        s += v * v;
+    // squared norms, a warp per row, four rows at a time (one round trip to
+    // memory for all of them; float atomics on one word take turns)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i0 = warp; i0 < m; i0 += 4 * nw) {
+      float s[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = i0 + r * nw;
+        s[r] = 0.0f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int j = lane + 32 * h;
+          const float v = (i < m && j < n) ? static_cast<float>(load_int(a.A, a.dtype, (long long)i * a.lda + j)) : 0.0f;
+          s[r] += v * v;
+        }
       }
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
-      if (lane == 0) bits[i] = F(0.5) * log2(max(s, F(1)));
+      for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[r] += __shfl_xor_sync(kFull, s[r], off);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (lane == 0 && i0 + r * nw < m) st.sq[i0 + r * nw] = s[r];
     }
   }
-  if (threadIdx.x == 0) bits[m] = log2(max(static_cast<F>(count), F(1)));
   __syncthreads();
 }
 
-// Number of primes for that bound, plus a sign bit and a margin, into
-// *needed, and the total row exponent of floating-point inputs into *esum;
-// row_e holds the row exponents and widths (2 m words).  The count is defined in binary64, whose
-// logarithms and sums are long chains on a slow pipe (the larger part of a
-// small call: 3 x 12 took 16.4 us a call with them).  The block therefore
-// sums the bits in binary32 first, whose error is below kNear of a prime
-// (at most 33 sums of at most 1100 bits for up to 32 primes: 2e-3 bits, 7e-5
-// primes, plus the norms' 1e-5), and redoes it in binary64 only when a count
-// boundary is that close.  row_bits: m + 1 words of shared scratch, bits32:
-// m + 1.  Ends with a barrier.
-__device__ inline void scale_and_count_primes(const SingleArgs& a, int m, double count, double* row_bits,
-                                              float* bits32, int* row_e, int* nonfinite, int* needed, int* esum) {
+// Number of primes for |det_R(A)| <= C(n,m) prod_i ||row_i||_2 (Hadamard's
+// inequality for every minor), plus a sign bit and a margin, into st.needed,
+// and the total row exponent into st.esum.  The count is defined in binary64,
+// whose logarithms and sums are long chains on a slow pipe: the block forms it
+// in binary32, whose error is below kNear of a prime (at most 33 sums of at
+// most 1100 bits for up to 32 primes: 2e-3 bits, 7e-5 primes, plus the norms'
+// 1e-5), and in binary64 only when a count boundary is that close.  Ends with
+// a barrier.
+__device__ inline void count_primes(const SingleArgs& a, int m, double count, RowStats& st) {
   constexpr float kNear = 1e-3f;
   const bool fp = is_fp_dtype(a.dtype);
-  if (fp) {
-    if (threadIdx.x == 0) *nonfinite = 0;
-    __syncthreads();
-    fp_row_scales(a.A, a.dtype, m, a.n, a.lda, row_e, nonfinite);
-    __syncthreads();
+  for (int i = threadIdx.x; i <= m; i += blockDim.x) {
+    if (i == m) st.bits[m] = log2f(fmaxf(static_cast<float>(count), 1.0f));
+    else if (fp) st.bits[i] = st.zero(i) ? 0.0f : static_cast<float>(st.width(i)) + 0.5f * log2f((float)a.n);
+    else st.bits[i] = 0.5f * log2f(fmaxf(st.sq[i], 1.0f));
   }
-  hadamard_bits<float>(a, m, count, row_e, bits32);
+  __syncthreads();
   float est = 0.0f;
-  int es = 0;
-  for (int i = 0; i <= m; ++i) est += bits32[i];
-  if (fp)
-    for (int i = 0; i < m; ++i) es += row_e[i];
+  for (int i = 0; i <= m; ++i) est += st.bits[i];
   const float q = (est + 2.0f) * (1.0f / 30.99f);
   int k = static_cast<int>(ceilf(q));
   if (fabsf(q - rintf(q)) <= kNear || !(q < 1e6f)) {  // the same in every thread
-    hadamard_bits<double>(a, m, count, row_e, row_bits);
-    double bits = row_bits[m];
-    for (int i = 0; i < m; ++i) bits += row_bits[i];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (fp) {
+      for (int i = threadIdx.x; i < m; i += blockDim.x)
+        st.bits64[i] = st.zero(i) ? 0.0 : static_cast<double>(st.width(i)) + 0.5 * log2(static_cast<double>(a.n));
+    } else {
+      for (int i = warp; i < m; i += nw) {
+        double s = 0.0;
+        for (int j = lane; j < a.n; j += 32) {
+          const double v = static_cast<double>(load_int(a.A, a.dtype, (long long)i * a.lda + j));
+          s += v * v;
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+        if (lane == 0) st.bits64[i] = 0.5 * log2(fmax(s, 1.0));
+      }
+    }
+    if (threadIdx.x == 0) st.bits64[m] = log2(fmax(count, 1.0));
+    __syncthreads();
+    double bits = st.bits64[m];
+    for (int i = 0; i < m; ++i) bits += st.bits64[i];
     k = static_cast<int>(ceil((bits + 2.0) / 30.99));
   }
   if (threadIdx.x == 0) {
-    *needed = k < 1 ? 1 : k;
-    *esum = es;
-    if (fp && *nonfinite) atomicExch(&a.hdr->status, RADIC_EINVAL);  // an entry is not finite
+    int es = 0;
+    if (fp)
+      for (int i = 0; i < m; ++i) es += st.exponent(i);
+    st.needed = k < 1 ? 1 : k;
+    st.esum = es;
+    if (st.nonfinite) atomicExch(&a.hdr->status, RADIC_EINVAL);  // an entry is not finite
   }
   __syncthreads();
 }
 
 // (T A mod p) in Montgomery form into As (column-major, column stride cs,
 // padding rows zero) for the prime mp: T = L U with L unit lower and U unit
-// upper triangular, entries from a hash of (slot, row, column).  Rows of U A
-// and of L (U A) are independent sums, so each product is one pass of the
-// block over the m n entries.  With alt_sign, odd columns are negated (the
-// column parities of Eq. (1)).  tri: m x m words, rows: 2 m n words of shared
-// scratch; row_e as from scale_and_count_primes.
-__device__ inline void stage_prime(const SingleArgs& a, int m, int cs, int slot, const Mont& mp, const int* row_e,
-                                   uint32_t* tri, uint32_t* rows, uint32_t* As, bool alt_sign) {
+// upper triangular, entries from a hash of (slot, row, column).  With
+// alt_sign, odd columns are negated (the column parities of Eq. (1)).  tri:
+// m x m words, rows: 2 m n words of shared scratch.
+__device__ inline void stage_prime(const SingleArgs& a, int m, int cs, int slot, const Mont& mp, const RowStats& st,
+                                   const KeptEntries& keep, uint32_t* tri, uint32_t* rows, uint32_t* As,
+                                   bool alt_sign) {
   const int n = a.n, mn = m * n;
   const bool fp = is_fp_dtype(a.dtype);
   uint32_t* ua = rows + mn;
@@ -383,27 +422,38 @@ __device__ inline void stage_prime(const SingleArgs& a, int m, int cs, int slot,
     const uint32_t r = static_cast<uint32_t>(h >> 33);  // 31 bits
     tri[idx] = r >= mp.p ? r - mp.p : r;
   }
-  for (int idx = threadIdx.x; idx < mn; idx += blockDim.x) {
+#pragma unroll
+  for (int k = 0; k < kKeepModp; ++k) {
+    const int idx = threadIdx.x + k * blockDim.x;
+    if (idx < mn) rows[idx] = fp ? fp_residue(keep.f[k], st.exponent(idx / n), mp) : int_residue(keep.v[k], mp.p);
+  }
+  for (int idx = threadIdx.x + kKeepModp * blockDim.x; idx < mn; idx += blockDim.x) {
     const int i = idx / n, j = idx - i * n;
     const long long at = (long long)i * a.lda + j;
-    rows[idx] = fp ? fp_residue(load_fp(a.A, a.dtype, at), row_e[i], mp)
+    rows[idx] = fp ? fp_residue(load_fp(a.A, a.dtype, at), st.exponent(i), mp)
                    : int_residue(load_int(a.A, a.dtype, at), mp.p);
   }
   __syncthreads();
+  // x + sum of u_l v_l over [l0, l1): two products per reduction
+  auto dot = [&](uint32_t x, const uint32_t* u, const uint32_t* v, int l0, int l1) {
+    int l = l0;
+    for (; l + 1 < l1; l += 2) {
+      const uint64_t t = static_cast<uint64_t>(u[l]) * v[l * n] + static_cast<uint64_t>(u[l + 1]) * v[(l + 1) * n];
+      x = add_mod(x, redc(t, mp.p, mp.pinv), mp.p);
+    }
+    if (l < l1) x = add_mod(x, mmul(u[l], v[l * n], mp), mp.p);
+    return x;
+  };
   for (int idx = threadIdx.x; idx < mn; idx += blockDim.x) {
     const int i = idx / n, j = idx - i * n;
-    uint32_t acc = rows[idx];
-    for (int l = i + 1; l < m; ++l) acc = add_mod(acc, mmul(tri[i * m + l], rows[l * n + j], mp), mp.p);
-    ua[idx] = acc;
+    ua[idx] = dot(rows[idx], tri + i * m, rows + j, i + 1, m);
   }
   __syncthreads();
   for (int idx = threadIdx.x; idx < n * cs; idx += blockDim.x) {
     const int j = idx / cs, i = idx - j * cs;
     uint32_t v = 0u;
     if (i < m) {
-      v = ua[i * n + j];
-      for (int l = 0; l < i; ++l) v = add_mod(v, mmul(tri[i * m + l], ua[l * n + j], mp), mp.p);
-      v = mmul(v, mp.r2, mp);
+      v = mmul(dot(ua[i * n + j], tri + i * m, ua + j, 0, i), mp.r2, mp);
       if (alt_sign && (j & 1)) v = neg_mod(v, mp.p);
     }
     As[idx] = v;
@@ -421,12 +471,13 @@ __device__ inline int stage_modp(const SingleArgs& a, const ModpSmem& sm, int m,
   build_binom(sm.binom, n, m);
   if (threadIdx.x < kMaxPrimes && base + (int)threadIdx.x < kWidePrimes)
     sm.mont[threadIdx.x] = make_mont(base + threadIdx.x);
-  scale_and_count_primes(a, m, static_cast<double>(sm.binom[n * (m + 1) + m]), sm.row_bits, sm.bits32, sm.row_e,
-                         &sm.misc[2], &sm.misc[0], &sm.misc[1]);
-  *needed = sm.misc[0];
-  const int K = max(0, min(min(sm.misc[0], kWidePrimes) - base, kMaxPrimes));
+  KeptEntries keep;
+  row_stats(a, m, *sm.stats, keep);
+  count_primes(a, m, static_cast<double>(sm.binom[n * (m + 1) + m]), *sm.stats);
+  *needed = sm.stats->needed;
+  const int K = max(0, min(min(*needed, kWidePrimes) - base, kMaxPrimes));
   for (int k = 0; k < K; ++k)
-    stage_prime(a, m, cs, k, sm.mont[k], sm.row_e, sm.tri, sm.rows, sm.As + (size_t)k * n * cs, false);
+    stage_prime(a, m, cs, k, sm.mont[k], *sm.stats, keep, sm.tri, sm.rows, sm.As + (size_t)k * n * cs, false);
   return K;
 }
 
@@ -533,6 +584,7 @@ __device__ inline void crt_write(radic_result* out, const uint32_t* res, int K, 
   uint32_t v[kMaxPrimes];
 #pragma unroll
   for (int i = 0; i < kMaxPrimes; ++i) {
+    if (i >= K) break;
     const Mont mp = make_mont(i);
     uint32_t acc = 0u;  // value of the digits so far modulo p
 #pragma unroll
@@ -577,6 +629,7 @@ __device__ inline void crt_write(radic_result* out, const uint32_t* res, int K, 
 // of the primes, gives the sign.  (Written serially, with an exponentiation
 // per digit and a limb-by-limb Horner rule, this took 245 us for 15 primes;
 // by a warp but with 64-bit divisions still 44 us.)
+static_assert(kMaxN <= 64, "two entries of a row per lane");
 static_assert(RADIC_WIDE_LIMBS == 32 && kWidePrimes == 32, "one lane per limb and prime; kAhead divides it");
 
 // x + carry-in from the lane below until no lane carries; lane 31's carry is lost.
@@ -677,11 +730,11 @@ __device__ inline void finish_modp(const SingleArgs& a, const ModpSmem& sm, uint
         for (int k = 0; k < K; ++k) a.wide[a.prime_base + k] = t[k];
         if (a.prime_base == 0) {
           a.wide[kWidePrimes] = static_cast<uint32_t>(needed);
-          a.wide[kWidePrimes + 1] = static_cast<uint32_t>(sm.misc[1]);
+          a.wide[kWidePrimes + 1] = static_cast<uint32_t>(sm.stats->esum);
           a.wide[kWidePrimes + 2] = static_cast<uint32_t>(__ldcg(&a.hdr->status));
         }
       } else {
-        crt_write(a.out, t, K, needed, __ldcg(&a.hdr->status), a.total, sm.misc[1]);
+        crt_write(a.out, t, K, needed, __ldcg(&a.hdr->status), a.total, sm.stats->esum);
       }
     }
   }

@@ -252,17 +252,15 @@ __device__ __noinline__ void subtree_pivoting(const uint32_t* __restrict__ As, c
 }
 
 // Shared-memory layout: binom | n x CS residues | 2 x (m x n) scratch rows |
-// m x m triangular factors | row bounds | row exponents | counts | block sum.
+// m x m triangular factors | row statistics | last-block flag | block sum.
 struct SubtreeSmem {
   uint64_t* binom;
   uint32_t* As;
   uint32_t* rows;
   uint32_t* tri;
-  double* row_bits;
-  float* bits32;
-  int* row_e;
-  int* misc;                 // primes the bound needs, total row exponent, non-finite flag, last-block flag
-  unsigned long long* sum;   // the block's residue sum
+  RowStats* stats;
+  int* last;
+  unsigned long long* sum;  // the block's residue sum
   size_t bytes;
   __host__ __device__ SubtreeSmem(unsigned char* base, int n, int m) {
     size_t off = 0;
@@ -275,10 +273,8 @@ struct SubtreeSmem {
     As = reinterpret_cast<uint32_t*>(base + take((size_t)n * ((m + 3) / 4 * 4) * 4));
     rows = reinterpret_cast<uint32_t*>(base + take(2 * (size_t)m * n * 4));
     tri = reinterpret_cast<uint32_t*>(base + take((size_t)m * m * 4));
-    row_bits = reinterpret_cast<double*>(base + take((size_t)(m + 1) * 8));
-    bits32 = reinterpret_cast<float*>(base + take((size_t)(m + 1) * 4));
-    row_e = reinterpret_cast<int*>(base + take((size_t)m * 8));
-    misc = reinterpret_cast<int*>(base + take(16));
+    stats = reinterpret_cast<RowStats*>(base + take(sizeof(RowStats)));
+    last = reinterpret_cast<int*>(base + take(16));
     sum = reinterpret_cast<unsigned long long*>(base + take(16));
     bytes = off;
   }
@@ -293,12 +289,13 @@ __global__ void __launch_bounds__(kMaxThreadsModp, G == 6 ? 3 : 4) k_modp_subtre
   const int kp = blockIdx.y;
   if (threadIdx.x == 0) *sm.sum = 0ull;
   build_binom(sm.binom, n, M);
-  scale_and_count_primes(a, M, static_cast<double>(sm.binom[n * bs + M]), sm.row_bits, sm.bits32, sm.row_e,
-                         &sm.misc[2], &sm.misc[0], &sm.misc[1]);
-  const int needed = sm.misc[0], K = min(needed, (int)gridDim.y);
+  KeptEntries keep;
+  row_stats(a, M, *sm.stats, keep);
+  count_primes(a, M, static_cast<double>(sm.binom[n * bs + M]), *sm.stats);
+  const int needed = sm.stats->needed, K = min(needed, (int)gridDim.y);
   if (kp >= K) return;  // a prime the bound does not need
   const Mont mp = make_mont(kp);
-  stage_prime(a, M, CS, kp, mp, sm.row_e, sm.tri, sm.rows, sm.As, true);
+  stage_prime(a, M, CS, kp, mp, *sm.stats, keep, sm.tri, sm.rows, sm.As, true);
 
   const int lane = threadIdx.x & 31;
   const unsigned long long wpb = blockDim.x / 32;
@@ -375,10 +372,10 @@ __global__ void __launch_bounds__(kMaxThreadsModp, G == 6 ? 3 : 4) k_modp_subtre
   if (threadIdx.x == 0) {
     if (*sm.sum) atomicAdd(&a.residue_sums[kp], *sm.sum);
     __threadfence();
-    sm.misc[3] = atomicAdd(&a.hdr->ticket[0], 1u) == gridDim.x * (unsigned)K - 1u;
+    *sm.last = atomicAdd(&a.hdr->ticket[0], 1u) == gridDim.x * (unsigned)K - 1u;
   }
   __syncthreads();
-  if (!sm.misc[3]) return;
+  if (!*sm.last) return;
   // the last block: residues of det_R (the common sign (-1)^(r + m) of Eq. (1)
   // that the folded column parities leave), then the reconstruction
   if (threadIdx.x < 32) {
@@ -391,12 +388,12 @@ __global__ void __launch_bounds__(kMaxThreadsModp, G == 6 ? 3 : 4) k_modp_subtre
     }
     const int status = __ldcg(&a.hdr->status);
     if (a.wide_out) {
-      wide_crt_warp(res, K, needed, sm.misc[1], status, a.total, a.wide_out);
+      wide_crt_warp(res, K, needed, sm.stats->esum, status, a.total, a.wide_out);
     } else {
       uint32_t all[kMaxPrimes];
 #pragma unroll
       for (int k = 0; k < kMaxPrimes; ++k) all[k] = __shfl_sync(kFull, res, k);
-      if (lane == 0) crt_write(a.out, all, K, needed, status, a.total, sm.misc[1]);
+      if (lane == 0) crt_write(a.out, all, K, needed, status, a.total, sm.stats->esum);
     }
   }
 }
