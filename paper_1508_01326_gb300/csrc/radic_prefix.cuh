@@ -587,12 +587,6 @@ __device__ __forceinline__ void leaf_column(const T* __restrict__ As, int col, c
   z[0] *= alpha;
 }
 
-// Sum over the aligned group of lp lanes (lp a power of two).
-__device__ __forceinline__ double group_sum(double x, int lp) {
-  for (int off = 1; off < lp; off <<= 1) x += __shfl_xor_sync(kFull, x, off);
-  return x;
-}
-
 // Leaf phase of one prefix without per-leaf output: the k later columns are
 // taken LB at a time (q, q+1, ...).  For each block, the leaves whose other
 // D-1 columns lie before the block read those columns' z from the buffer
@@ -606,10 +600,8 @@ __device__ __forceinline__ double group_sum(double x, int lp) {
 //
 // kCoop: the buffer already holds every column's z (written by the lanes
 // sharing the prefix, see prefix_leaves); the block's columns are read from
-// it instead of being reduced here.  kSeq: the lanes' column sums are added
-// up over the group and the first lane takes them, column by column, as one
-// lane alone would.
-template <typename T, int M, int D, int CS, bool kCoop, bool kSeq, bool kB>
+// it instead of being reduced here.
+template <typename T, int M, int D, int CS, bool kCoop, bool kB>
 __device__ __forceinline__ void prefix_leaves_blocked(const T* __restrict__ As, int v, int k, const T (&W)[D][M - D],
                                                       const int (&idx)[M], T alpha, const ZBuf<T, D>& zb, bool act,
                                                       int sub, int lp, PrefixAcc<T>& acc, T& zmax,
@@ -714,11 +706,7 @@ __device__ __forceinline__ void prefix_leaves_blocked(const T* __restrict__ As, 
       bsum += cs[b];
       babs += ca[b];
     }
-    if constexpr (kSeq) {
-      bsum = group_sum(bsum, lp);
-      babs = group_sum(babs, lp);
-    }
-    if (act && (!kSeq || sub == 0)) {
+    if (act) {
       acc.add_column(bsum, babs);
       lb.term_abs(babs);
     }
@@ -727,6 +715,36 @@ __device__ __forceinline__ void prefix_leaves_blocked(const T* __restrict__ As, 
       for (int b = 0; b < LB; ++b) {
         if (q + b < k) zb.put(q + b, z[b]);
       }
+    }
+  }
+}
+
+// The leaves whose last column is q, all columns being in the buffer: signed
+// and absolute sums, in the order of the blocked form with one column per step.
+template <typename T, int D>
+__device__ __forceinline__ void column_leaves(const ZBuf<T, D>& zb, int q, T& cs, T& ca) {
+  T z[D];
+  zb.get(q, z);
+  cs = ca = T(0);
+  if constexpr (D == 2) {
+#pragma unroll 2
+    for (int q2 = 0; q2 < q; ++q2) {
+      T y[2];
+      zb.get(q2, y);
+      leaf_add(det2(y, z), cs, ca);
+    }
+  } else {
+    for (int q2 = 1; q2 < q; ++q2) {
+      T y2[3], w[3], s2 = T(0);
+      zb.get(q2, y2);
+      cross3(y2, z, w);
+#pragma unroll 2
+      for (int q1 = 0; q1 < q2; ++q1) {
+        T y1[3];
+        zb.get(q1, y1);
+        leaf_add(dot3(y1, w), s2, ca);
+      }
+      cs += s2;
     }
   }
 }
@@ -844,11 +862,15 @@ __device__ __noinline__ void prefix_minors_f64(const double* __restrict__ As, co
   }
 }
 
-// kSeq (binary64): lanes that share a prefix reproduce the error bound of one
-// lane working it alone bit for bit, whatever their number: the columns'
-// (norm, radius) pairs and the column sums of |terms| enter its sums one
-// column after the other (bounds are binary32 sums, whose rounding otherwise
-// depends on how many lanes share the prefix).
+// kSeq (binary64): lanes that share a prefix take whole columns, both for the
+// Schur complements and for the leaves that end in a column, so every sum over
+// leaves is formed by one lane in the order of one lane alone, and the error
+// bound takes the columns' (norm, radius) pairs and sums of |terms| one after
+// the other: the bound's bits do not depend on the number of lanes (bounds are
+// binary32 sums).  Splitting each column's leaves instead costs a reduction
+// over the group per column, ten dependent binary64 additions (5 x 16: 35 us
+// against 25).  The redo flag returned covers the lane's own columns: binary64
+// has no redo.
 template <typename T, int M, int D, int CS, bool kTerms, bool kRedo = true, bool kSeq = false>
 __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const uint64_t* binom, int n, int v,
                                               const int (&c)[M - D], const T (&W)[D][M - D], const int (&idx)[M],
@@ -897,42 +919,52 @@ __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const ui
                                      ts, nan_out);
   } else {
     if constexpr (kSeq) {
-      // Two phases as below; each column's (norm, radius) goes to the buffer
-      // slot of the lane after the group's first (8 bytes per column, free
-      // when lp > 1), from which every lane takes all of them in order.
-      static_assert(sizeof(T) == 8, "one slot entry holds two binary32 numbers");
-      const ZBuf<T, D> zg = zb.shifted(-sub);
+      static_assert(sizeof(T) == 8, "a buffer entry holds two binary32 numbers per plane");
       if (D == 2 && lp == 1) {
         // one lane, depth 2: columns and leaves in one pass (two passes
         // measured 11% slower on 256 x 6 x 28)
-        prefix_leaves_blocked<T, M, D, CS, false, false>(As, v, k, W, idx, alpha, zb, act, 0, 1, acc, zmax, lb);
-      } else if (lp == 1) {
-        for (int q = 0; q < k; ++q) {
-          T z[D];
-          leaf_column<T, M, D, CS>(As, v + 1 + q, W, idx, alpha, z, zmax, lb);
-          zg.put(q, z);
-        }
+        prefix_leaves_blocked<T, M, D, CS, false>(As, v, k, W, idx, alpha, zb, act, 0, 1, acc, zmax, lb);
+        __syncwarp();
       } else {
-        const ZBuf<T, D> ng = zg.shifted(1);
+        // a column's norm, radius and sum of |terms| go to the entry of the
+        // lane after the group's first, free when lp > 1
+        const ZBuf<T, D> zg = zb.shifted(-sub), ng = zg.shifted(1);
+        auto norms = [&](int q) { return reinterpret_cast<float2*>(&ng.p[q * ng.stride]); };
+        auto terms = [&](int q) {
+          if constexpr (D == 2) return reinterpret_cast<float*>(&ng.p[q * ng.stride]) + 2;
+          else return reinterpret_cast<float*>(&ng.p[q * ng.stride + ng.plane]);
+        };
         for (int q = sub; q < k; q += lp) {
           T z[D];
           float nr[2];
           leaf_column<T, M, D, CS>(As, v + 1 + q, W, idx, alpha, z, zmax, lb, nr);
           zg.put(q, z);
-          *reinterpret_cast<float2*>(&ng.p[q * ng.stride]) = make_float2(nr[0], nr[1]);
+          if (lp == 1) lb.poly.add(nr[0], nr[1]);
+          else *norms(q) = make_float2(nr[0], nr[1]);
         }
-        zmax = group_max(zmax, lp);
         __syncwarp();
-        for (int q = 0; q < k; ++q) {
-          const float2 nr = *reinterpret_cast<const float2*>(&ng.p[q * ng.stride]);
-          lb.poly.add(nr.x, nr.y);
+        // columns cost more the later they are: the lanes take them in turns
+        // of alternating direction
+        for (int q0 = 0; q0 < k; q0 += lp) {
+          const int q = q0 + ((q0 & lp) ? lp - 1 - sub : sub);
+          if (q < k) {
+            T cs, ca;
+            column_leaves<T, D>(zg, q, cs, ca);
+            if (act) acc.add_column(cs, ca);
+            if (lp == 1) lb.term_abs(ca);
+            else *terms(q) = mag(ca);
+          }
+        }
+        __syncwarp();
+        if (lp > 1) {
+          for (int q = 0; q < k; ++q) {
+            const float2 nr = *norms(q);
+            lb.poly.add(nr.x, nr.y);
+            lb.pabs += *terms(q);
+          }
+          __syncwarp();  // the buffer is rewritten by the group's next prefix
         }
       }
-      if (D == 3 || lp > 1) {
-        __syncwarp();
-        prefix_leaves_blocked<T, M, D, CS, true, true>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
-      }
-      __syncwarp();  // the buffer is rewritten by the group's next prefix
     } else if constexpr (D == 3) {
       // Two phases.  The lp lanes sharing the prefix split its column
       // reductions: lane `sub` reduces the columns q = sub (mod lp) into the
@@ -950,10 +982,10 @@ __device__ __forceinline__ bool prefix_leaves(const T* __restrict__ As, const ui
       zmax = group_max(zmax, lp);
       group_combine(lb.poly, lp);
       __syncwarp();
-      prefix_leaves_blocked<T, M, D, CS, true, false>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
+      prefix_leaves_blocked<T, M, D, CS, true>(As, v, k, W, idx, alpha, zg, act, sub, lp, acc, zmax, lb);
       __syncwarp();  // the buffer is rewritten by the group's next prefix
     } else {
-      prefix_leaves_blocked<T, M, D, CS, false, false>(As, v, k, W, idx, alpha, zb, act, sub, lp, acc, zmax, lb);
+      prefix_leaves_blocked<T, M, D, CS, false>(As, v, k, W, idx, alpha, zb, act, sub, lp, acc, zmax, lb);
     }
   }
   bool bad = false;
