@@ -558,8 +558,9 @@ __device__ __forceinline__ void warp_reduce_ff(Ff& t, Ff& ta) {
 
 // Block-wide fixed-order reduction of float-float lane totals, a count and
 // the lanes' error bounds (binary64), the totals entirely on the binary32
-// pipe (binary64 runs at 1/64 of its rate): warp trees, then the warps'
-// totals in warp order.  The result is valid in thread 0.  `scratch` holds
+// pipe (binary64 runs at 1/64 of its rate): warp trees, then a tree over the
+// warps' totals (one after the other they were four dependent binary64 merges,
+// twice per call).  The result is valid in thread 0.  `scratch` holds
 // kScratchWords * (blockDim.x / 32) binary64 words.
 constexpr int kScratchWords = 5;
 __device__ inline void block_reduce_ff(Ff& t, Ff& ta, long long& count, double& bnd, double* scratch) {
@@ -582,22 +583,32 @@ __device__ inline void block_reduce_ff(Ff& t, Ff& ta, long long& count, double& 
     ws[3] = bnd;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Ff s, sa;
-    long long cnt = 0;
-    double b = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      const double* wv = scratch + kScratchWords * w;
+  if (warp == 0) {  // the warps' totals, by a tree again (at most eight warps)
+    t = ta = Ff();
+    count = 0;
+    bnd = 0.0;
+    if (lane < nw) {
+      const double* wv = scratch + kScratchWords * lane;
       const float* fv = reinterpret_cast<const float*>(wv);
-      s.merge(Ff{fv[0], fv[1]});
-      sa.merge(Ff{fv[2], fv[3]});
-      cnt += __double_as_longlong(wv[2]);
-      b += wv[3];
+      t = Ff{fv[0], fv[1]};
+      ta = Ff{fv[2], fv[3]};
+      count = __double_as_longlong(wv[2]);
+      bnd = wv[3];
     }
-    t = s;
-    ta = sa;
-    count = cnt;
-    bnd = b;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+      if (off < nw) {
+        Ff o, oa;
+        o.hi = __shfl_xor_sync(kFull, t.hi, off);
+        o.lo = __shfl_xor_sync(kFull, t.lo, off);
+        oa.hi = __shfl_xor_sync(kFull, ta.hi, off);
+        oa.lo = __shfl_xor_sync(kFull, ta.lo, off);
+        t.merge(o);
+        ta.merge(oa);
+        count += __shfl_xor_sync(kFull, count, off);
+        bnd += shfl_xor_d(bnd, off);
+      }
+    }
   }
 }
 
@@ -626,24 +637,30 @@ __device__ inline void block_reduce_dd(Dd& acc, double& abs_sum, long long& coun
     ws[4] = bnd;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Dd t;
-    double ab = 0.0, b = 0.0;
-    long long cnt = 0;
-    for (int w = 0; w < nw; ++w) {
-      const double* wv = scratch + kScratchWords * w;
-      Dd o;
-      o.hi = wv[0];
-      o.lo = wv[1];
-      t.merge(o);
-      ab += wv[2];
-      cnt += __double_as_longlong(wv[3]);
-      b += wv[4];
+  if (warp == 0) {  // the warps' totals, by a tree again (at most eight warps)
+    acc = Dd();
+    abs_sum = bnd = 0.0;
+    count = 0;
+    if (lane < nw) {
+      const double* wv = scratch + kScratchWords * lane;
+      acc.hi = wv[0];
+      acc.lo = wv[1];
+      abs_sum = wv[2];
+      count = __double_as_longlong(wv[3]);
+      bnd = wv[4];
     }
-    acc = t;
-    abs_sum = ab;
-    count = cnt;
-    bnd = b;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+      if (off < nw) {
+        Dd o;
+        o.hi = shfl_xor_d(acc.hi, off);
+        o.lo = shfl_xor_d(acc.lo, off);
+        acc.merge(o);
+        abs_sum += shfl_xor_d(abs_sum, off);
+        count += __shfl_xor_sync(kFull, count, off);
+        bnd += shfl_xor_d(bnd, off);
+      }
+    }
   }
 }
 
