@@ -325,8 +325,13 @@ int make_plan_uncached(int m, int n, int mode, const radic_options* o, unsigned 
   // one contiguous run of about C(n,m)/K ranks.  K is the number of resident
   // processors of a full-occupancy grid, so every processor gets one task and
   // no SM waits on a tail; an explicit ranks_per_task overrides the run length.
-  const unsigned long long cap = (unsigned long long)sms * per_sm;
   if (mapping == RADIC_MAP_PREFIX) return plan_prefix(pl, d, sms, per_sm, units, p);
+  // Floating-point groups: the split is that of 512 threads per SM whatever
+  // the kernel's registers leave resident (groups of 32: 384), because the
+  // binary32 sums of bounds round per run; the blocks beyond those resident even out the tail
+  // (17 x 22: 485 us against 508 with runs for the resident blocks).
+  const unsigned long long cap =
+      (unsigned long long)sms * (mapping == RADIC_MAP_GROUP && mode != kModeExact ? 512 / pl.threads : per_sm);
   const unsigned long long per_block =
       (mapping == RADIC_MAP_THREAD) ? (unsigned long long)pl.threads : (unsigned long long)(pl.threads / pl.group);
   unsigned long long L = (unsigned long long)d.ranks_per_task;

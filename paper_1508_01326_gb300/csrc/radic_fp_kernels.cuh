@@ -424,23 +424,23 @@ __device__ __forceinline__ T group_det(T (&x)[G], int m, int sub, int seg, T& gm
 // What bounds it: shuffles (two for the pivot row's entry, one for its radius
 // per step) and the binary64 pipe, one multiply-add per step and warp however
 // few lanes are rows.  12 x 20 (126 thousand minors): 751 us with every minor
-// eliminated on its own, 405 us now (the pipe 58% busy while the SMs are, which
+// eliminated on its own, 393 us now (the pipe 58% busy while the SMs are, which
 // is 76% of the time: later minors of dictionary order change more columns).
 template <typename T, int G, bool kGrowth>
 struct GroupLu {
   T l[G];
   float al[G], rl[G];
-  int p[G];
+  unsigned p[(G + 3) / 4];  // a byte each
   // lane j: state after step j
   T det_s, gmax_s;
   float rel_s, pr_s;
   unsigned alive_s;  // rows left
   int flags_s;       // bit 0 parity of the row permutation, bit 1 a pivot's enclosure reached zero
 
-  // Eliminates the minor whose columns c[first..m-1] are new; As: staged
-  // matrix (column stride m).  `first` is the same in every group of the warp.
-  // Returns det; bnd, bad and gmax are valid in every lane of the group.
-  __device__ __forceinline__ T run(const T* __restrict__ As, const int (&c)[G], int first, int m, int sub, T& gmax,
+  // Eliminates the minor whose columns first..m-1 are new; lane j holds column
+  // c_j in cs.  As: staged matrix (column stride m).  `first` is the same in
+  // every group of the warp.  Returns det; bnd, bad and gmax are valid in every lane of the group.
+  __device__ __forceinline__ T run(const T* __restrict__ As, int cs, int first, int m, int sub, T& gmax,
                                    float& bnd, bool& bad, float u_in) {
     constexpr float u = static_cast<float>(BoundTraits<T>::u);
     constexpr float c_div = static_cast<float>(BoundTraits<T>::c_div);
@@ -459,9 +459,6 @@ struct GroupLu {
       alive = m == 32 ? kFull : (1u << m) - 1u;
       flags = 0;
     }
-    int cs = 0;  // lane j: column c_j
-#pragma unroll
-    for (int j = 0; j < G; ++j) cs = sub == j ? c[j] : cs;
     bool last_open = false;
     // one copy of the column body for every j (a copy per column measured half
     // of its time in instruction fetches)
@@ -473,9 +470,10 @@ struct GroupLu {
 #pragma unroll
       for (int k = 0; k < G - 1; ++k) {
         if (k >= j) break;  // the same in every lane of the warp
-        const T uj = __shfl_sync(kFull, x, p[k], G);
-        const float ru = __shfl_sync(kFull, rx, p[k], G);
-        const float old = mag(x), au = __shfl_sync(kFull, old, p[k], G);  // |uj| as its own lane forms it
+        const int pk = p[k / 4] >> (8 * (k % 4));  // the shuffles take it modulo G
+        const T uj = __shfl_sync(kFull, x, pk, G);
+        const float ru = __shfl_sync(kFull, rx, pk, G);
+        const float old = mag(x), au = __shfl_sync(kFull, old, pk, G);  // |uj| as its own lane forms it
         x = fma(-l[k], uj, x);
         // rx += al ru + (au + ru) rl + u (al au + old)
         rx += fmaf(u, fmaf(al[k], au, old), fmaf(al[k], ru, __fmul_rn(au + ru, rl[k])));
@@ -517,7 +515,8 @@ struct GroupLu {
           l[k] = lj;
           al[k] = aj;
           rl[k] = rj;
-          p[k] = pk;
+          const int sh = 8 * (k % 4);
+          p[k / 4] = (p[k / 4] & ~(0xffu << sh)) | ((unsigned)pk << sh);
         }
       }
       if (sub == j) {
@@ -538,10 +537,12 @@ struct GroupLu {
   }
 };
 
-// Groups of 16: four blocks of 128 threads per SM (the plan's ranks per group
-// follow from it).  Groups of 32 hold twice the multipliers and would spill.
+// Registers: four blocks of 128 threads per SM for groups of 16, three for
+// groups of 32, which hold twice the multipliers (four would spill most of
+// them; unconstrained they take 248 and two blocks fit: 18 x 21, 333 blocks,
+// 96 us against 64).
 template <typename T, int G, bool kMixed, bool kTerms>
-__global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(SingleArgs a) {
+__global__ void __maxnreg__(G == 16 ? 128 : 168) k_fp_group(SingleArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = a.n, m = a.m;
   FpSmem<T> sm(smem_raw, n, m, m);
@@ -556,6 +557,7 @@ __global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(Sin
 
   const int lane = threadIdx.x & 31, sub = lane & (G - 1), seg = lane / G;
   constexpr int kSegs = 32 / G;
+  constexpr unsigned segbits = G == 32 ? kFull : (1u << G) - 1u;
   // a block's warps take tasks a grid apart: minors late in dictionary order
   // change more columns each, and neighbouring tasks on one SM would make it
   // the last to finish
@@ -579,8 +581,13 @@ __global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(Sin
     const bool tact = task < a.tasks;
     const unsigned long long q0 = qbase + (tact ? task : 0ull) * L;
     const unsigned long long q1 = min(q0 + L, qlim);
-    int c[G];
-    unrank_dyn<G>(q0, n, m, sm.binom, m + 1, c);
+    int cs = 0;  // column c_sub
+    {
+      int c[G];
+      unrank_dyn<G>(q0, n, m, sm.binom, m + 1, c);
+#pragma unroll
+      for (int j = 0; j < G; ++j) cs = sub == j ? c[j] : cs;
+    }
     Ff run;
     float run_abs = 0.0f, run_bnd = 0.0f;
     int first = 0;  // first column that changed since the previous minor
@@ -593,19 +600,23 @@ __global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(Sin
       if constexpr (kTerms) {
         T x[G];
 #pragma unroll
-        for (int j = 0; j < G; ++j) x[j] = (j < m && sub < m) ? sm.As[c[j] * m + sub] : T(0);
+        for (int j = 0; j < G; ++j) {
+          const int cj = __shfl_sync(kFull, cs, j, G);
+          x[j] = (j < m && sub < m) ? sm.As[cj * m + sub] : T(0);
+        }
         det = group_det<T, G>(x, m, sub, seg, gmax);
       } else {
-        det = lu.run(sm.As, c, first, m, sub, gmax, b, bad, uin);
-        if (bad && !kMixed) {  // Hadamard's inequality alone
+        det = lu.run(sm.As, cs, first, m, sub, gmax, b, bad, uin);
+        if (!kMixed && __any_sync(kFull, bad)) {  // Hadamard's inequality alone
+          const float nrm = sub < m ? static_cast<float>(sm.colnorm[cs]) : 1.0f;
           float h = 1.0f;
-#pragma unroll
-          for (int j = 0; j < G; ++j)
-            if (j < m) h *= static_cast<float>(sm.colnorm[c[j]]);
-          b = mag(det) * 1.0000002f + h;
+          for (int j = 0; j < m; ++j) h *= __shfl_sync(kFull, nrm, j, G);
+          if (bad) b = mag(det) * 1.0000002f + h;
         }
       }
-      if (sign_negative_dyn<G>(c, m)) det = -det;
+      // the sign of sign_negative
+      const unsigned odd = (__ballot_sync(kFull, sub < m && (cs & 1)) >> (seg * G)) & segbits;
+      if ((m * (m + 1) / 2 + m + __popc(odd)) & 1) det = -det;
       bool flag = false;
       if constexpr (kMixed) flag = mixed_flag<T>(det, gmax, thr) || bad;
       const bool lead = act && sub == 0;
@@ -652,8 +663,12 @@ __global__ void __launch_bounds__(kMaxThreadsFp, G == 16 ? 2 : 1) k_fp_group(Sin
           run_bnd = 0.0f;
         }
       }
-      const int changed = q + 1 < q1 ? successor_dyn<G>(c, n, m) : m - 1;
-      if constexpr (!kTerms) first = __reduce_min_sync(kFull, changed);  // over the warp's groups
+      // successor: the last column that can still move does, the later ones follow it
+      const unsigned can = (__ballot_sync(kFull, sub < m && cs < n - m + sub) >> (seg * G)) & segbits;
+      const int pos = can != 0u ? 31 - __clz(can) : 0, cp = __shfl_sync(kFull, cs, pos, G);
+      const bool more = q + 1 < q1;
+      if (more && sub >= pos && sub < m) cs = cp + 1 + sub - pos;
+      if constexpr (!kTerms) first = __reduce_min_sync(kFull, more ? pos : m - 1);  // over the warp's groups
     }
     if constexpr (!kTerms) {
       if constexpr (kMixed) {
