@@ -22,6 +22,7 @@ LIB_PATH = os.path.join(HERE, "libradic.so")
 SOURCES = [
     "radic_api.cu",
     "radic_fp64.cu",
+    "radic_fp64_share.cu",
     "radic_mixed.cu",
     "radic_pair.cu",
     "radic_modp.cu",

@@ -200,8 +200,39 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
     if (run > maxrun) run = maxrun > 0 ? maxrun : 1;
     t.lanes[v] = lp;
     t.run[v] = run;
-    t.task_start[v] = start;
     start += (t.count[v] + groups * run - 1) / (groups * run);
+  }
+  // Binary64 depth 3: the lanes of a group can factor a prefix each and then
+  // share the leaves of one after the other (prefix_group), so that runs of up
+  // to lp prefixes cost one elimination where every lane used to repeat the
+  // prefix's own.  Runs grow to one task per resident warp by the cost of a
+  // shared prefix's leaves (a lane's share, and per column what the group does
+  // together).  Taken if it halves the tasks at least: 10 x 20 850 -> 341 us,
+  // 9 x 20 432 -> 226, 8 x 20 178 -> 131.  (Grown by number alone, whatever
+  // the leaves cost, 7 x 20 and 8 x 20 were 1.35 times slower than before.)
+  if (pl.mode == kModeFp64 && D == 3 && m >= 7 && d.ranks_per_task == 0) {
+    const double red = (double)m * P * P;
+    double total = 0.0;
+    auto leaves = [&](int v) { return (cost[v] - red) / t.lanes[v] + 30.0 * (n - 1 - v); };
+    for (int v = t.v_lo; v <= t.v_hi; ++v) total += (double)t.count[v] * (red + t.lanes[v] * leaves(v));
+    const double share = total / (double)lanes;
+    unsigned long long runs[kMaxN], tasks = 0;
+    for (int v = t.v_lo; v <= t.v_hi; ++v) {
+      const unsigned long long lp = t.lanes[v], groups = 32 / lp, maxrun = (t.count[v] + groups - 1) / groups;
+      const unsigned long long fit = share > red ? (unsigned long long)((share - red) / leaves(v)) : 0ull;
+      runs[v] = std::max(t.run[v], std::min({lp, fit, maxrun}));
+      tasks += (t.count[v] + groups * runs[v] - 1) / (groups * runs[v]);
+    }
+    if (2 * tasks <= start) {
+      t.share = 1;
+      std::copy(runs + t.v_lo, runs + t.v_hi + 1, t.run + t.v_lo);
+    }
+  }
+  start = 0;
+  for (int v = t.v_lo; v <= t.v_hi; ++v) {
+    const unsigned long long chunk = 32ull / t.lanes[v] * t.run[v];
+    t.task_start[v] = start;
+    start += (t.count[v] + chunk - 1) / chunk;
   }
   if (t.v_hi + 1 < kMaxN) t.task_start[t.v_hi + 1] = start;
   if (t.v_hi < t.v_lo) start = 0;

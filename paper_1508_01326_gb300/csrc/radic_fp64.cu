@@ -26,6 +26,7 @@ const void* prefix_kernel(bool terms) {
 
 const void* pick(const SinglePlan& p, bool terms) {
   if (p.mapping == RADIC_MAP_PREFIX) {
+    if (p.ptab.share && !terms) return fp64_shared_kernel(p.m);
     switch (p.m) {
       case 3: return p.depth == 2 ? prefix_kernel<3, 2>(terms) : nullptr;
       case 4: return p.depth == 3 ? prefix_kernel<4, 3>(terms) : prefix_kernel<4, 2>(terms);

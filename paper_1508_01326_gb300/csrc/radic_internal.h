@@ -89,6 +89,7 @@ struct PrefixTable {
   unsigned long long task_start[kMaxN];    // first task index of group v
   int lanes[kMaxN];                        // lanes sharing one prefix in group v (1..32, power of 2)
   int dynamic;                             // warps draw later tasks from the header counter
+  int share;                               // a lane group factors a prefix per lane (binary64, depth 3)
 };
 
 // Launch plan of one single-matrix call (computed identically by
@@ -170,6 +171,7 @@ enum : int { kModpDet = 0, kModpWide = 1, kModpTerms = 2 };
 
 // Occupancy helpers filled in by the arithmetic files.
 int blocks_per_sm_fp64(const SinglePlan& p);
+const void* fp64_shared_kernel(int m);  // prefix mapping, depth 3, m 7..10
 int blocks_per_sm_mixed(const SinglePlan& p);
 int blocks_per_sm_pair(const SinglePlan& p);
 int blocks_per_sm_modp(const SinglePlan& p, int use);

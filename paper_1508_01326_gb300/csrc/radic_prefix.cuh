@@ -1067,6 +1067,74 @@ __device__ __forceinline__ bool prefix_one(const T* __restrict__ As, const uint6
   }
 }
 
+// A lane group's next prefixes: lane `sub` factors prefix r + sub of group v,
+// then the lp lanes work the leaves of one after the other, each taking the
+// factorisation from the lane that has it (65 shuffles at m = 8 against the
+// elimination, some hundreds of binary64 instructions, which every lane repeats
+// when the group shares one prefix at a time).  10 x 20, where nearly every
+// prefix is shared by 32 lanes: 850 -> 341 us.  What is left is latency: the
+// columns of a prefix follow each other, a few dependent binary64 operations
+// and a group reduction each, with two warps per scheduler.  Sums and bounds
+// only, no terms.
+template <int M, int D, int CS>
+__device__ __forceinline__ void prefix_group(const double* __restrict__ As, const uint64_t* binom, int n, int v,
+                                             unsigned long long r, unsigned long long r1, unsigned long long cnt,
+                                             int nj, const ZBuf<double, D>& zb, double thr, int lane, int sub, int lp,
+                                             PrefixAcc<double>& acc, const TermsSink& ts, float uin) {
+  constexpr int P = M - D;
+  static_assert(M <= 16 && P <= 8, "row numbers in four bits, columns in eight");
+  double W[D][P], prod, gmax;
+  float rW[D][P], rel;
+  uint64_t rows = 0, cols = 0;
+  int neg_bad;
+  {
+    int c[P], idx[M];
+    if constexpr (P > 1) {
+      int head[P - 1];
+      unrank<P - 1>(r + sub < cnt ? r + sub : 0ull, v, binom, M + 1, head);
+#pragma unroll
+      for (int j = 0; j < P - 1; ++j) c[j] = head[j];
+    }
+    c[P - 1] = v;
+    bool neg, bad;
+    prefix_factor_b<double, M, D, CS>(As, c, W, rW, idx, prod, gmax, neg, rel, bad, uin);
+    neg_bad = (neg ? 1 : 0) | (bad ? 2 : 0);
+#pragma unroll
+    for (int i = 0; i < M; ++i) rows |= (uint64_t)idx[i] << (4 * i);
+#pragma unroll
+    for (int j = 0; j < P; ++j) cols |= (uint64_t)c[j] << (8 * j);
+  }
+  for (int j = 0; j < nj; ++j) {
+    const bool act = r + j < r1;
+    if (!__any_sync(kFull, act)) break;
+    const int src = lane - sub + j;
+    double Wj[D][P];
+    float rWj[D][P];
+    int idx[M], c[P];
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+#pragma unroll
+      for (int i = 0; i < P; ++i) {
+        Wj[d][i] = __shfl_sync(kFull, W[d][i], src);
+        rWj[d][i] = __shfl_sync(kFull, rW[d][i], src);
+      }
+    const double pj = __shfl_sync(kFull, prod, src), gj = __shfl_sync(kFull, gmax, src);
+    const int nb = __shfl_sync(kFull, neg_bad, src);
+    const uint64_t rj = __shfl_sync(kFull, rows, src), cj = __shfl_sync(kFull, cols, src);
+#pragma unroll
+    for (int i = 0; i < M; ++i) idx[i] = (int)(rj >> (4 * i)) & 15;
+#pragma unroll
+    for (int i = 0; i < P; ++i) c[i] = (int)(cj >> (8 * i)) & 255;
+    PrefixErr<float> pe;
+    pe.kappa = 0.0f;
+    pe.rel_alpha = __shfl_sync(kFull, rel, src);
+    pe.bad = (nb & 2) != 0;
+    prefix_leaves<double, M, D, CS, false, false>(As, binom, n, v, c, Wj, idx, pj, gj, (nb & 1) != 0, zb, thr, act, sub,
+                                                  lp, acc, ts, pe, rWj, uin);
+    acc.end_prefix();
+  }
+}
+
 // Head sharing: the prefixes whose first H = m-D-1 columns (the head) agree
 // share those H elimination steps.  The head is factored once with
 // prefix_factor at depth D+1 (W1 = -L21 L11^{-1} for the D+1 rows left);
@@ -1352,7 +1420,10 @@ __host__ __device__ constexpr int prefix_min_blocks() {
                                        : (std::is_same<T, ff>::value ? RADIC_PREFIX_MIN_BLOCKS_FF : 1);
 }
 
-template <typename T, int M, int D, bool kMixed, bool kTerms>
+// kShare: runs of several prefixes per lane group (prefix_group).  Its own
+// kernel: the shuffles of prefix_group cost launches of single-prefix tasks 1
+// to 5% (8 x 32, 7 x 30).
+template <typename T, int M, int D, bool kMixed, bool kTerms, bool kShare = false>
 __global__ void __launch_bounds__(128, prefix_min_blocks<T>()) k_fp_prefix(SingleArgs a, PrefixTable tab) {
   static_assert(M > D, "the prefix needs at least one column");
   constexpr int P = M - D;
@@ -1408,6 +1479,13 @@ __global__ void __launch_bounds__(128, prefix_min_blocks<T>()) k_fp_prefix(Singl
     const unsigned long long groups = 32 / lp;
     const unsigned long long r0 = (t - tab.task_start[v]) * groups * runlen + (unsigned long long)grp * runlen;
     const unsigned long long r1 = min(r0 + runlen, cnt);
+    if constexpr (kShare) {
+      for (unsigned long long it = 0; it < runlen; it += lp)
+        prefix_group<M, D, CS>(sm.As, sm.binom, n, v, r0 + it, r1, cnt, (int)min((unsigned long long)lp, runlen - it),
+                               zb, thr, lane, sub, lp, acc, ts, uin);
+      t = tab.dynamic ? __shfl_sync(kFull, t_next, 0) : t_next;
+      continue;
+    }
     constexpr int H = P > 1 ? P - 1 : 1;
     int head[H];  // first P-1 prefix columns, a (P-1)-subset of {0..v-1}
     if constexpr (P > 1) unrank<P - 1>(r0 < cnt ? r0 : 0ull, v, sm.binom, bs, head);
