@@ -25,13 +25,15 @@
 // into z),
 //   g_q,i = dL / dz_i(x_q) = sum over T not holding i of +- P[T] R[rest],
 // the sign that of bringing the rows (T, i, rest) into order.  P and R follow
-// from column to column by one exterior product with z (R by taking z(x_q)
-// out again: R_q = (1 - z) ^ R_{q-1}), G 2^(G-1) multiply-adds each.  Taking
-// columns out keeps the rounding of the larger sums it starts from, so R is
-// built from the last column to the first, kept at two columns on the way, and
-// taken up from there again (with one start alone the gradient's error was
-// 2.1 times that of the sums over two columns, in both arithmetics).  Then
-// column q receives alpha (-1)^q [W^T; I] g_q, and the head's own columns
+// from column to column by one exterior product with z, G 2^(G-1) multiply-adds
+// each: P from the first column on, R from the last column back.  Both only
+// ever take columns in.  (R could also follow P forwards, taking z(x_q) out
+// again, but what is left keeps the rounding of the sums that held it: with one
+// column r times the others the gradient's error grew like r^2 2^-53.)  The two
+// run in opposite directions, so R is kept once per segment of columns on the
+// way back, and each segment is built again from there, every column's R
+// stored, when P comes to it.  Then column q receives
+// alpha (-1)^q [W^T; I] g_q, and the head's own columns
 // alpha [L A^{-1} - A^{-1} Q W | -A^{-1} Q]^T with Q = sum_q (-1)^q x_T(q) g_q^T.
 // A head thus costs O(k G (2^G + m)) operations for its k later columns,
 // whatever the number C(k, G) of its minors.
@@ -40,8 +42,8 @@
 // SM, whether or not all its lanes are used) or, in pairs, dependent binary32
 // chains at 8 warps per SM.  G trades the number of heads, C(n-G, m-G),
 // against the cost of a column (bwd_plan).  256 matrices of 6 x 28, binary64:
-// 0.57 ms with G = 4, the pipe 72% busy (6.0 ms with G = 2 and lanes grouped by
-// equal v, the pipe 83% busy).
+// 0.60 ms with G = 4 (6.0 ms with G = 2 and lanes grouped by equal v, the pipe
+// 83% busy; 0.57 ms with R taken forwards, see above).
 //
 // Lanes take heads in colexicographic order (by last column v, then in
 // dictionary order), so that a warp is full whatever the sizes of the groups
@@ -80,6 +82,7 @@ struct BwdArgs {
   long long lda, stride;  // row stride, matrix stride (elements)
   int batch, m, n;
   int chunks;             // blocks per matrix
+  int seg;                // columns per segment of the suffix sums (head kernel; even)
   unsigned long long total;
   double* slots;          // batch x chunks x m x n (chunks > 1)
   const double* grad_out;
@@ -448,9 +451,8 @@ __device__ __forceinline__ void append_column(T (&P)[1 << G], const T (&z)[G]) {
   }
 }
 
-// R <- (1 + z) ^ R (kAdd: z becomes the first column of R's sequences) or
-// (1 - z) ^ R (takes the first column z out again).
-template <typename T, int G, bool kAdd, int MAXS, int SET>
+// R <- (1 + z) ^ R: z becomes the first column of R's sequences.
+template <typename T, int G, int MAXS, int SET>
 __device__ __forceinline__ void first_column(T (&R)[1 << G], const T (&z)[G]) {
   if constexpr (SET >= 1) {
     constexpr int size = bits_of(SET);
@@ -458,13 +460,13 @@ __device__ __forceinline__ void first_column(T (&R)[1 << G], const T (&z)[G]) {
 #pragma unroll
       for (int i = 0; i < G; ++i) {
         if ((SET >> i) & 1) {
-          const bool neg = (bits_of(SET & ((1 << i) - 1)) & 1) != (kAdd ? 0 : 1);
+          const bool neg = bits_of(SET & ((1 << i) - 1)) & 1;
           if constexpr (size == 1) R[SET] = R[SET] + signed_of(neg, z[i]);
           else R[SET] = fma(signed_of(neg, z[i]), R[SET ^ (1 << i)], R[SET]);
         }
       }
     }
-    first_column<T, G, kAdd, MAXS, SET - 1>(R, z);
+    first_column<T, G, MAXS, SET - 1>(R, z);
   }
 }
 
@@ -580,6 +582,19 @@ __device__ __noinline__ void singular_head(const double* Ab, long long lda, cons
   }
 }
 
+// Blocks per SM that the head kernel's registers allow (its launch bound).
+__host__ __device__ constexpr int bwd_resident(int m) { return m == 3 ? 4 : m == 4 ? 3 : 2; }
+// Words a lane stores per column of a segment: R without its full set, and z.
+__host__ __device__ constexpr int bwd_store_words(int G) { return (1 << G) - 2 + G; }
+// Fewest columns per segment: what fits bwd_resident blocks at n = 64.
+__host__ __device__ constexpr int bwd_min_segment(int G) { return G == 4 ? 4 : G == 3 ? 6 : 10; }
+// A warp's working memory: a segment's columns, or a singular head's two sets of
+// 2^m sums.
+__host__ __device__ inline size_t bwd_work_bytes(int m, int G, int seg) {
+  const size_t cols = (size_t)seg * bwd_store_words(G) * 32 * 8, sing = (size_t)2 * 8 << m;
+  return cols > sing ? cols : sing;
+}
+
 // Shared-memory layout of the head kernel.
 template <typename T>
 struct BwdSmem {
@@ -587,10 +602,9 @@ struct BwdSmem {
   T* As;
   double* tile0;    // tile of the singular heads
   T* tiles;         // one m x n tile per warp
-  double* scratch;  // 2^(m+1) words per warp
-  T* kept;          // R at two columns, 2^G - 2 sums each, lane by lane
+  unsigned char* work;  // bwd_work_bytes per warp
   size_t bytes;
-  __host__ __device__ BwdSmem(unsigned char* base, int n, int m, int G, int warps) {
+  __host__ __device__ BwdSmem(unsigned char* base, int n, int m, int G, int seg, int warps) {
     size_t off = 0;
     auto take = [&](size_t b) {
       const size_t o = off;
@@ -601,22 +615,22 @@ struct BwdSmem {
     As = reinterpret_cast<T*>(base + take((size_t)n * ((m + 1) / 2 * 2) * 8));
     tile0 = reinterpret_cast<double*>(base + take((size_t)m * n * 8));
     tiles = reinterpret_cast<T*>(base + take((size_t)warps * m * n * 8));
-    scratch = reinterpret_cast<double*>(base + take((size_t)warps * (16u << m)));
-    kept = reinterpret_cast<T*>(base + take((size_t)2 * ((1 << G) - 2) * warps * 32 * 8));
+    work = base + take((size_t)warps * bwd_work_bytes(m, G, seg));
     bytes = off;
   }
 };
 
 template <typename T, int M, int G>
-__global__ void __launch_bounds__(kBwdThreads, 2) k_backward_heads(BwdArgs a) {
-  constexpr int H = M - G, FULL = (1 << G) - 1;
+__global__ void __launch_bounds__(kBwdThreads, bwd_resident(M)) k_backward_heads(BwdArgs a) {
+  constexpr int H = M - G, FULL = (1 << G) - 1, kWords = bwd_store_words(G);
   constexpr int CS = ColStride<T, M>::value;
   static_assert(sizeof(T) == 8 && CS == (M + 1) / 2 * 2, "layout of BwdSmem");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = a.n, bs = M + 1;
   const int b = blockIdx.y, chunk = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  const BwdSmem<T> sm(smem_raw, n, M, G, wpb);
+  const BwdSmem<T> sm(smem_raw, n, M, G, a.seg, wpb);
+  unsigned char* const work = sm.work + (size_t)warp * bwd_work_bytes(M, G, a.seg);
   build_binom(sm.binom, n, M);
   const double* Ab = a.A + (long long)b * a.stride;
   for (int idx = threadIdx.x; idx < n * CS; idx += blockDim.x) {
@@ -695,7 +709,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_backward_heads(BwdArgs a) {
       int cs[H];
 #pragma unroll
       for (int j = 0; j < H; ++j) cs[j] = __shfl_sync(kFull, c[j], __ffs(sing) - 1);
-      singular_head<M, G>(Ab, a.lda, cs, n, sm.scratch + (size_t)warp * (2u << M), sm.tile0, lane);
+      singular_head<M, G>(Ab, a.lda, cs, n, reinterpret_cast<double*>(work), sm.tile0, lane);
     }
     // below, a singular or repeated head runs with non-finite or unwanted
     // values that `use` replaces by zeros
@@ -731,42 +745,30 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_backward_heads(BwdArgs a) {
         for (int d = 0; d < G; ++d) z[d] = -z[d];
       }
     };
-    // pass 1: the sums over all later columns; R[FULL] = L
-    T R[1 << G], P[1 << G];
+    // Segments of the later columns, last to first (step < 0, then 0): R[FULL] =
+    // L in the end.  Then first to last: each segment's R built again from its
+    // kept start (the first one's are still there), then the gradients of its
+    // columns (summed over the warp) and Q.
+    T R[1 << G], P[1 << G], L = T(0);
 #pragma unroll
     for (int S = 0; S <= FULL; ++S) R[S] = P[S] = T(0);
-    // kept at third points of the warp's columns
-    const int third = (n - col0 + 2) / 3, keep1 = col0 + third, keep2 = keep1 + third;
-    T* kept = sm.kept + threadIdx.x;
-    for (int col = n - 1; col >= col0; --col) {
-      if (col > v) {
-        T z[G];
-        schur(col, z);
-        first_column<T, G, true, G, FULL>(R, z);
-      }
-      if (col == keep1 || col == keep2) {
-#pragma unroll
-        for (int S = 1; S < FULL; ++S) kept[((col == keep1 ? 0 : FULL - 1) + S - 1) * kBwdThreads] = R[S];
-      }
-    }
-    const T L = R[FULL];
-    // pass 2: gradients of the later columns (summed over the warp) and Q
     T Q[H][G];
 #pragma unroll
     for (int i = 0; i < H; ++i)
 #pragma unroll
       for (int d = 0; d < G; ++d) Q[i][d] = T(0);
-    auto column = [&](int col, T (&val)[M]) {
+    // local memory, written and read once per segment
+    T kept[(kMaxN + bwd_min_segment(G) - 1) / bwd_min_segment(G)][FULL - 1];
+    T* store = reinterpret_cast<T*>(work) + lane;
+    auto column = [&](int col, int at, T (&val)[M]) {  // at: place in its segment
 #pragma unroll
       for (int i = 0; i < M; ++i) val[i] = T(0);
-      if (col == keep1 || col == keep2) {
-#pragma unroll
-        for (int S = 1; S < FULL; ++S) R[S] = kept[((col == keep1 ? 0 : FULL - 1) + S - 1) * kBwdThreads];
-      }
       if (col > v) {
         T z[G], g[G];
-        schur(col, z);
-        first_column<T, G, false, G - 1, FULL>(R, z);
+#pragma unroll
+        for (int S = 1; S < FULL; ++S) R[S] = store[(at * kWords + S - 1) * 32];
+#pragma unroll
+        for (int d = 0; d < G; ++d) z[d] = store[(at * kWords + FULL - 1 + d) * 32];
         contract<T, G>(P, R, g);
         append_column<T, G, G - 1, FULL>(P, z);
         const T* xc = As + col * CS;
@@ -793,26 +795,54 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_backward_heads(BwdArgs a) {
         unpermute<T, M>(w, idx, val);
       }
     };
-    if constexpr (std::is_same<T, ff>::value) {
-      // pairs: one column per warp sum (the column body is long; inlining it
-      // twice measured slower, with instruction-fetch stalls)
-      for (int col = col0; col < n; ++col) {
-        T va[M];
-        column(col, va);
-        warp_add_column<T, M>(va, Gw + col, n, lane);
-      }
-    } else {
-      for (int col = col0; col < n; col += 2) {  // binary64: two columns per warp sum
-        const bool two = col + 1 < n;
-        T va[M], vb[M];
-        column(col, va);
-        if (two) {
-          column(col + 1, vb);
-        } else {
+    const int last = (n - 1 - col0) / a.seg;
+#pragma unroll 1
+    for (int step = -last; step <= last; ++step) {
+      const int sg = step < 0 ? -step : step, a0 = col0 + sg * a.seg, a1 = min(n, a0 + a.seg);
+      if (step <= 0) {
 #pragma unroll
-          for (int i = 0; i < M; ++i) vb[i] = T(0);
+        for (int S = 1; S < FULL; ++S) kept[sg][S - 1] = R[S];
+      } else {
+#pragma unroll
+        for (int S = 1; S < FULL; ++S) R[S] = kept[sg][S - 1];
+      }
+#pragma unroll 1
+      for (int col = a1 - 1; col >= a0; --col) {
+        if (col <= v) continue;
+        T z[G];
+        schur(col, z);
+        if (step >= 0) {
+          T* at = store + (col - a0) * kWords * 32;
+#pragma unroll
+          for (int S = 1; S < FULL; ++S) at[(S - 1) * 32] = R[S];
+#pragma unroll
+          for (int d = 0; d < G; ++d) at[(FULL - 1 + d) * 32] = z[d];
         }
-        warp_add_columns2<T, M>(va, vb, Gw + col, n, lane, two);
+        first_column<T, G, G, FULL>(R, z);
+      }
+      if (step < 0) continue;
+      if (step == 0) L = R[FULL];
+      if constexpr (std::is_same<T, ff>::value) {
+        // pairs: one column per warp sum (the column body is long; inlining it
+        // twice measured slower, with instruction-fetch stalls)
+        for (int col = a0; col < a1; ++col) {
+          T va[M];
+          column(col, col - a0, va);
+          warp_add_column<T, M>(va, Gw + col, n, lane);
+        }
+      } else {
+        for (int col = a0; col < a1; col += 2) {  // binary64: two columns per warp sum
+          const bool two = col + 1 < a1;
+          T va[M], vb[M];
+          column(col, col - a0, va);
+          if (two) {
+            column(col + 1, col + 1 - a0, vb);
+          } else {
+#pragma unroll
+            for (int i = 0; i < M; ++i) vb[i] = T(0);
+          }
+          warp_add_columns2<T, M>(va, vb, Gw + col, n, lane, two);
+        }
       }
     }
     // head columns: alpha [L Ainv - Ainv Q W | -Ainv Q]^T, in pivot order row
@@ -904,7 +934,7 @@ const void* bwd_heads_kernel(int m, int G) {
 }
 
 struct BwdPlan {
-  int G = 0, chunks = 1;
+  int G = 0, chunks = 1, seg = 0;
 };
 
 // Subtree depth and blocks per matrix of the head kernel.  Estimate for every
@@ -923,7 +953,7 @@ BwdPlan bwd_plan(int batch, int m, int n, int sms) {
     const int H = m - G;
     const double ext = G * (double)(1 << (G - 1)) - G;
     const double head = m * (double)H * H + 2.0 * H * H * H + H * (G * (double)H + (double)G * H + 3.0 * m) + 40.0;
-    const double col = 2.0 * G * H + 3.0 * ext + G * (double)(1 << (G - 1)) + 2.0 * G * H + G + 10.0;
+    const double col = 3.0 * G * H + 3.0 * ext + G * (double)(1 << (G - 1)) + 2.0 * G * H + G + 10.0;
     double cols = 0.0, heads = 0.0;
     for (int v = H - 1; v <= n - 1 - G; ++v) {
       const double cnt = (double)binom_host(v, H - 1);
@@ -942,6 +972,17 @@ BwdPlan bwd_plan(int batch, int m, int n, int sms) {
       best.chunks = (int)std::max(1ll, std::min(std::min(by_work, want), 65535ll));
     }
   }
+  // Segments as long as the shared memory of the blocks that run together on an
+  // SM allows: a segment's columns are computed twice, but for the first's.
+  // (5000 matrices of 3 x 30, 16 columns and three blocks per SM 507 us, 12 and
+  // four 449; 64 of them, one block per SM, 12 columns 51 us, 24 45.)
+  const long long blocks = (long long)batch * best.chunks;
+  const int resident = (int)std::max(1ll, std::min<long long>((blocks + sms - 1) / sms, bwd_resident(m)));
+  const size_t room = std::min<size_t>(228 * 1024 / resident - 1024, 227 * 1024);
+  const int cols = n - (m - best.G);
+  best.seg = bwd_min_segment(best.G);
+  while (best.seg < cols && BwdSmem<double>(nullptr, n, m, best.G, best.seg + 2, kBwdThreads / 32).bytes <= room)
+    best.seg += 2;
   return best;
 }
 
@@ -1010,6 +1051,7 @@ int radic_det_backward_mode(const double* A, int batch, int m, int n, int64_t ld
   a.m = m;
   a.n = n;
   a.total = binom_host(n, m);
+  a.seg = 0;
   a.chunks = bwd_chunks(batch, a.total);
   a.slots = static_cast<double*>(workspace);
   a.grad_out = grad_out;
@@ -1019,8 +1061,9 @@ int radic_det_backward_mode(const double* A, int batch, int m, int n, int64_t ld
   if (m >= 3) {  // shared per head
     const BwdPlan p = bwd_plan(batch, m, n, device_sm_count());
     a.chunks = p.chunks;
+    a.seg = p.seg;
     k = (mode == RADIC_MODE_PAIR) ? bwd_heads_kernel<ff>(m, p.G) : bwd_heads_kernel<double>(m, p.G);
-    smem = BwdSmem<double>(nullptr, n, m, p.G, kBwdThreads / 32).bytes;
+    smem = BwdSmem<double>(nullptr, n, m, p.G, p.seg, kBwdThreads / 32).bytes;
   } else {
     k = bwd_kernel(m);
     smem = bwd_smem(m, n);
