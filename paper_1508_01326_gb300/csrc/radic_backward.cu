@@ -495,55 +495,38 @@ __device__ __forceinline__ void contract(const T (&P)[1 << G], const T (&R)[1 <<
 // Gradient of a head's subtree without elimination, by the whole warp, in
 // binary64 from the matrix in global memory: the same sums over sets of all M
 // rows, a prefix sum V that starts from the determinants of the head's columns
-// instead of 1, and suffix sums R over the later columns.  Serves heads with
-// an exactly zero pivot.  scratch: 2^(M+1) words of shared memory; G: the
-// block's gradient tile (shared-memory atomics).
+// instead of 1, and suffix sums R over the later columns, both taking columns
+// in only.  R is built from the last column back for as many columns at a time
+// as the working memory holds.  Serves heads with an exactly zero pivot.  work:
+// `arrays` (at least 4) arrays of 2^M words of shared memory; G: the block's
+// gradient tile (shared-memory atomics).
 template <int M, int GD>
 __device__ __noinline__ void singular_head(const double* Ab, long long lda, const int (&c)[M - GD], int n,
-                                           double* scratch, double* G, int lane) {
+                                           double* work, int arrays, double* G, int lane) {
   constexpr int H = M - GD, NS = 1 << M;
-  double* V = scratch;
-  double* R = scratch + NS;
-  auto entry = [&](int i, int col) {  // column parity of Eq. (1) folded in
-    const double x = Ab[(long long)i * lda + col];
-    return (col & 1) ? -x : x;
-  };
-  // E <- E + E ^ x (front: (1 - x) ^ E) for the sets of lo..hi rows, largest first
-  auto wedge = [&](double* E, int col, int lo, int hi, bool front) {
-    for (int size = hi; size >= lo; --size) {
-      for (int S = lane; S < NS; S += 32) {
-        if (__popc(S) != size) continue;
-        double acc = E[S];
-        int pos = 0;
-        for (int i = 0; i < M; ++i) {
-          if (!((S >> i) & 1)) continue;
-          const bool neg = front ? !(pos & 1) : ((size - 1 - pos) & 1);
-          const double t = entry(i, col) * E[S ^ (1 << i)];
-          acc += neg ? -t : t;
-          ++pos;
-        }
-        E[S] = acc;
-      }
-      __syncwarp();
-    }
-  };
-  // sum over the sets T without row i of +- V[T] R[rest], for every row i,
-  // into column `col` of the tile
-  auto scatter = [&](int col, bool neg) {
-    for (int i = 0; i < M; ++i) {
-      double s = 0.0;
-      for (int T = lane; T < NS; T += 32) {
-        if ((T >> i) & 1) continue;
-        const int rest = (NS - 1) ^ T ^ (1 << i);
-        int inv = __popc(T >> (i + 1)) + __popc(rest & ((1 << i) - 1));
-        for (int u = 0; u < M; ++u)
-          if ((rest >> u) & 1) inv += __popc(T >> (u + 1));
-        const double t = V[T] * R[rest];
-        s += (inv & 1) ? -t : t;
-      }
+  // to <- E + E ^ x, the column appended (front: E + x ^ E), for the sets of
+  // lo..hi rows; the others are copied.  Column parity of Eq. (1) folded in.
+  auto wedge = [&](const double* E, double* to, int col, int lo, int hi, bool front) {
+    double x[M];
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
-      if (lane == 0) atomicAdd(G + i * n + col, neg ? -s : s);
+    for (int i = 0; i < M; ++i) {
+      const double e = Ab[(long long)i * lda + col];
+      x[i] = (col & 1) ? -e : e;
+    }
+    for (int S = lane; S < NS; S += 32) {
+      const int size = __popc(S);
+      double acc = E[S];
+      if (size >= lo && size <= hi) {
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+          if ((S >> i) & 1) {
+            const int below = __popc(S & ((1 << i) - 1));
+            const bool neg = ((front ? below : size - 1 - below) & 1) != 0;
+            acc = fma(neg ? -x[i] : x[i], E[S ^ (1 << i)], acc);
+          }
+        }
+      }
+      to[S] = acc;
     }
     __syncwarp();
   };
@@ -551,34 +534,79 @@ __device__ __noinline__ void singular_head(const double* Ab, long long lda, cons
     for (int S = lane; S < NS; S += 32) E[S] = S == 0 ? 1.0 : 0.0;
     __syncwarp();
   };
+  // R over the columns from `col` on, into `to` (spare: another array)
+  auto suffix = [&](int col, double* to, double* spare) {
+    double *from = ((n - col) & 1) ? spare : to, *into = ((n - col) & 1) ? to : spare;
+    unit(from);
+    for (int q = n - 1; q >= col; --q) {
+      wedge(from, into, q, 1, GD, true);
+      double* t = from;
+      from = into;
+      into = t;
+    }
+  };
+  // sum over the sets T of `lo` rows or more, without row i, of +- V[T] R[rest],
+  // for every row i, into column `col` of the tile.  The sign is that of (T, i,
+  // rest): T before the other rows (its row numbers less 0, 1, ...), then i
+  // before those of `rest` below it.
+  auto scatter = [&](const double* V, const double* R, int lo, int hi, int col, bool neg) {
+    double s[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) s[i] = 0.0;
+    for (int T = lane; T < NS; T += 32) {
+      const int size = __popc(T);
+      if (size < lo || size > hi) continue;
+      const double vt = V[T];
+      const int moved = __popc(T & 0xaa) + size * (size - 1) / 2;
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        if (!((T >> i) & 1)) {
+          const int rest = (NS - 1) ^ T ^ (1 << i);
+          const bool odd = ((moved + __popc(rest & ((1 << i) - 1))) & 1) != 0;
+          s[i] = fma(odd ? -vt : vt, R[rest], s[i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s[i] += __shfl_xor_sync(kFull, s[i], off);
+      if (lane == 0) atomicAdd(G + i * n + col, neg ? -s[i] : s[i]);
+    }
+    __syncwarp();
+  };
   const bool common = (M * (M + 1) / 2 + M) & 1;  // (-1)^(r+s) without the column parities
-  // suffix sums over all later columns, sets of up to GD rows
-  unit(R);
-  for (int col = c[H - 1] + 1; col < n; ++col) wedge(R, col, 1, GD, false);
+  double *V = work, *next = work + NS, *R = work + 2 * NS;
+  auto append = [&](int col, int lo, int hi) {
+    wedge(V, next, col, lo, hi, false);
+    double* t = V;
+    V = next;
+    next = t;
+  };
   // head column j: the determinants of the other head columns (sets of H-1
   // rows) against the sums over GD columns; column j moves past H-1-j columns
+  suffix(c[H - 1] + 1, R, R + NS);
   for (int j = 0; j < H; ++j) {
     unit(V);
     int size = 0;
     for (int t = 0; t < H; ++t) {
       if (t == j) continue;
-      wedge(V, c[t], 1, ++size, false);
+      ++size;
+      append(c[t], 1, size);
     }
-    for (int S = lane; S < NS; S += 32)
-      if (__popc(S) != H - 1) V[S] = 0.0;
-    __syncwarp();
-    scatter(c[j], common ^ ((c[j] & 1) != 0) ^ (((H - 1 - j) & 1) != 0));
+    scatter(V, R, H - 1, H - 1, c[j], common ^ ((c[j] & 1) != 0) ^ (((H - 1 - j) & 1) != 0));
   }
   // later columns: V starts from the head's own determinants
   unit(V);
-  for (int t = 0; t < H; ++t) wedge(V, c[t], 1, t + 1, false);
-  for (int S = lane; S < NS; S += 32)
-    if (__popc(S) != H) V[S] = 0.0;
-  __syncwarp();
-  for (int col = c[H - 1] + 1; col < n; ++col) {
-    wedge(R, col, 1, GD, true);
-    scatter(col, common ^ ((col & 1) != 0));
-    wedge(V, col, H + 1, M - 1, false);
+  for (int t = 0; t < H; ++t) append(c[t], 1, t + 1);
+  for (int a0 = c[H - 1] + 1; a0 < n; a0 += arrays - 2) {
+    const int a1 = min(n, a0 + arrays - 2);
+    suffix(a1, R + (a1 - 1 - a0) * NS, next);  // R after column a1-1, then after each one before
+    for (int col = a1 - 1; col > a0; --col) wedge(R + (col - a0) * NS, R + (col - 1 - a0) * NS, col, 1, GD, true);
+    for (int col = a0; col < a1; ++col) {
+      scatter(V, R + (col - a0) * NS, H, M - 1, col, common ^ ((col & 1) != 0));
+      append(col, H + 1, M - 1);
+    }
   }
 }
 
@@ -588,10 +616,10 @@ __host__ __device__ constexpr int bwd_resident(int m) { return m == 3 ? 4 : m ==
 __host__ __device__ constexpr int bwd_store_words(int G) { return (1 << G) - 2 + G; }
 // Fewest columns per segment: what fits bwd_resident blocks at n = 64.
 __host__ __device__ constexpr int bwd_min_segment(int G) { return G == 4 ? 4 : G == 3 ? 6 : 10; }
-// A warp's working memory: a segment's columns, or a singular head's two sets of
-// 2^m sums.
+// A warp's working memory: a segment's columns, or a singular head's arrays of
+// 2^m words.
 __host__ __device__ inline size_t bwd_work_bytes(int m, int G, int seg) {
-  const size_t cols = (size_t)seg * bwd_store_words(G) * 32 * 8, sing = (size_t)2 * 8 << m;
+  const size_t cols = (size_t)seg * bwd_store_words(G) * 32 * 8, sing = (size_t)4 * 8 << m;
   return cols > sing ? cols : sing;
 }
 
@@ -709,7 +737,8 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_resident(M)) k_backward_heads
       int cs[H];
 #pragma unroll
       for (int j = 0; j < H; ++j) cs[j] = __shfl_sync(kFull, c[j], __ffs(sing) - 1);
-      singular_head<M, G>(Ab, a.lda, cs, n, reinterpret_cast<double*>(work), sm.tile0, lane);
+      singular_head<M, G>(Ab, a.lda, cs, n, reinterpret_cast<double*>(work),
+                          (int)(bwd_work_bytes(M, G, a.seg) / (8u << M)), sm.tile0, lane);
     }
     // below, a singular or repeated head runs with non-finite or unwanted
     // values that `use` replaces by zeros
