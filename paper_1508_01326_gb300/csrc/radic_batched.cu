@@ -106,9 +106,10 @@ double default_task_cost(double total_cost, int batch) {
 // Minors one lane works for one unit of a head-shared task at most (a single
 // prefix, up to C(n-m+D, D) minors, is never split): a head's whole subtree
 // holds up to C(n-m+1, D+1) minors, and the longest unit sets the kernel's
-// critical path.  Scales with the task cost.
-unsigned long long segment_minors(double task_cost) {
-  return (unsigned long long)(4096.0 * std::min(1.0, task_cost / kTaskCost));
+// critical path.  In binary64 it scales with the task cost; the other tiers
+// keep it, because their bounds and sums of |terms| round per lane total.
+unsigned long long segment_minors(int tier, double task_cost) {
+  return (unsigned long long)(4096.0 * (tier == kModeFp64 ? std::min(1.0, task_cost / kTaskCost) : 1.0));
 }
 
 // Splits the last columns v = u+1 .. n-1-D of the heads with last column u
@@ -201,7 +202,7 @@ int make_tasks(radic_batch_plan& pl, int b, int tier, const radic_batch_tuning* 
     t.shared = 1;
     for (int u = H - 1; u <= n - 2 - D; ++u) {
       const unsigned long long cnt = binom_host(u, H - 1);
-      for (const auto& sg : head_segments(n, D, u, segment_minors(lane_cost))) {
+      for (const auto& sg : head_segments(n, D, u, segment_minors(tier, lane_cost))) {
         const double c = head_cost(m, D, n, sg.first, sg.second);
         const unsigned long long run = task_run(cnt, c, lane_cost, tier);
         t.vlo = sg.first;
