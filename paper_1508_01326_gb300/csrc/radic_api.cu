@@ -160,47 +160,85 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
   }
   const unsigned long long lanes = (unsigned long long)sms * per_sm * pl.threads;
   const double per_lane = total_cost / (double)lanes / 4.0;  // about four tasks per warp
-  unsigned long long start = 0;
-  for (int v = t.v_lo; v <= t.v_hi; ++v) {
-    // Lanes per prefix: a prefix with many candidate columns costs far more
-    // than a lane's share of the launch (the leaves grow like C(k, D)), so
-    // its column reductions and leaves are split over LP lanes of the warp,
-    // each of which repeats the factorisation.  LP is the smallest power of
-    // two that brings a lane's cost down to a target near the mean per-lane
-    // work.
+  const double red = (double)m * P * P;  // elimination, repeated by every lane that shares a prefix
+  // Smallest power of two of lanes that brings a lane's cost down to `target`.
+  auto lanes_for = [&](int v, double target) {
     int lp = 1;
-    if (d.lanes_per_prefix > 0) {
-      lp = d.lanes_per_prefix;
-    } else if (D == 3 || (pl.mode == kModeFp64 && m >= 4)) {
-      // Depth 3 (its leaves grow like C(k, 3)), and binary64 depth 2, whose
-      // small launches otherwise leave most SMs idle behind one lane's chain
-      // of binary64 operations (5 x 16: 5 blocks on 152 SMs).  In the other
-      // modes splitting depth-2 prefixes measured slower.  Target with binary32 elimination: 1.4
-      // times the mean lane work when that is large, three times when the
-      // launch is small and the repeated factorisations would dominate.
-      // Binary64 and pair leaves keep their pipes busy, so there the balance
-      // of the warps' shares matters more than the repeated work: the mean
-      // itself.  (Measured on the shapes of prefix_auto_depth, warps drawing
-      // tasks from the shared counter.)
-      // Binary64 depth 2: the mean over one warp per scheduler, which is what
-      // keeps the binary64 pipe busy (over all resident lanes every group of a
-      // 6 x 24 matrix was split, and the repeated factorisations doubled its
-      // time).
-      const double mean = D == 2 ? total_cost / ((double)sms * 128.0) : 4.0 * per_lane;
-      const double tf = (pl.mode == kModeMixed) ? (mean >= 1000.0 ? 1.4 : 3.0) : 1.0;
-      const double target = tf * mean;
-      const double red = (double)m * P * P, split = cost[v] - red;
-      while (lp < 32 && red + split / lp > target) lp *= 2;
-    }
+    while (lp < 32 && red + (cost[v] - red) / lp > target) lp *= 2;
+    return lp;
+  };
+  auto run_for = [&](int v, int lp) {
     const unsigned long long groups = 32 / lp;  // lane groups per warp
-    double r = per_lane * lp / cost[v];
+    const double r = per_lane * lp / cost[v];
     unsigned long long run = r < 1.0 ? 1ull : (unsigned long long)r;
     if (d.ranks_per_task > 0) run = (unsigned long long)d.ranks_per_task;
     const unsigned long long maxrun = (t.count[v] + groups - 1) / groups;
     if (run > maxrun) run = maxrun > 0 ? maxrun : 1;
+    return run;
+  };
+  // Lanes per prefix: a prefix with many candidate columns costs far more
+  // than a lane's share of the launch (the leaves grow like C(k, D)), so
+  // its column reductions and leaves are split over several lanes of the
+  // warp, each of which repeats the factorisation.
+  const bool seq = pl.mode == kModeFp64 && D == 2 && m >= 4;
+  double target = 0.0;
+  if (D == 3) {
+    // Near the mean per-lane work.  With binary32 elimination: 1.4
+    // times the mean lane work when that is large, three times when the
+    // launch is small and the repeated factorisations would dominate.
+    // Binary64 and pair leaves keep their pipes busy, so there the balance
+    // of the warps' shares matters more than the repeated work: the mean
+    // itself.  (Measured on the shapes of prefix_auto_depth, warps drawing
+    // tasks from the shared counter.)
+    const double mean = 4.0 * per_lane;
+    target = (pl.mode == kModeMixed ? (mean >= 1000.0 ? 1.4 : 3.0) : 1.0) * mean;
+  } else if (seq) {
+    // Binary64 depth 2, whose small launches otherwise leave most SMs idle
+    // behind one lane's chain of binary64 operations (5 x 16: 5 blocks on 152
+    // SMs).  In the other modes splitting depth-2 prefixes measured slower.
+    // The mean over one warp per scheduler, which is what keeps the binary64
+    // pipe busy, as long as the tasks fit one wave of warps.
+    target = total_cost / ((double)sms * 128.0);
+    double work, longest, most = 0.0;  // of the plan with target tau, in cost units
+    auto tasks_for = [&](double tau) {
+      unsigned long long tasks = 0;
+      work = longest = 0.0;
+      for (int v = t.v_lo; v <= t.v_hi; ++v) {
+        const int lp = lanes_for(v, tau);
+        const unsigned long long run = run_for(v, lp), chunk = 32ull / lp * run, k = (t.count[v] + chunk - 1) / chunk;
+        const double c = (double)run * (red + (cost[v] - red) / lp);
+        tasks += k;
+        work += (double)k * c;
+        longest = std::max(longest, c);
+        most = std::max(most, cost[v]);
+      }
+      return tasks;
+    };
+    if (tasks_for(target) > (unsigned long long)sms * per_sm * (pl.threads / 32) && target < 4.0 * red) {
+      // A mean near or below the elimination itself splits every prefix as far
+      // as it goes and repeats the elimination for nothing: the target with
+      // the least estimate instead.  A cost unit takes an SM 10 ns and a lone
+      // warp 30, a task as much as 95 units (fitted to 250 plans of m = 4..6,
+      // n = 6..63).  6 x 23 on 32 lanes throughout 99 us, one lane each 71,
+      // now 33; 5 x 26 41, 82, 27.
+      double best = 0.0;
+      for (double tau = std::max(target, 1.05 * red);; tau *= 1.15) {
+        const double tasks = (double)tasks_for(tau), time = 10.0 * (work + 95.0 * tasks) / sms + 30.0 * longest;
+        if (best == 0.0 || time < best) {
+          best = time;
+          target = tau;
+        }
+        if (tau >= most) break;
+      }
+    }
+  }
+  unsigned long long start = 0;
+  for (int v = t.v_lo; v <= t.v_hi; ++v) {
+    const int lp = d.lanes_per_prefix > 0 ? d.lanes_per_prefix : D == 3 || seq ? lanes_for(v, target) : 1;
     t.lanes[v] = lp;
-    t.run[v] = run;
-    start += (t.count[v] + groups * run - 1) / (groups * run);
+    t.run[v] = run_for(v, lp);
+    const unsigned long long chunk = 32ull / lp * t.run[v];
+    start += (t.count[v] + chunk - 1) / chunk;
   }
   // Binary64 depth 3: the lanes of a group can factor a prefix each and then
   // share the leaves of one after the other (prefix_group), so that runs of up
@@ -211,7 +249,6 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
   // 9 x 20 432 -> 226, 8 x 20 178 -> 131.  (Grown by number alone, whatever
   // the leaves cost, 7 x 20 and 8 x 20 were 1.35 times slower than before.)
   if (pl.mode == kModeFp64 && D == 3 && m >= 7 && d.ranks_per_task == 0) {
-    const double red = (double)m * P * P;
     double total = 0.0;
     auto leaves = [&](int v) { return (cost[v] - red) / t.lanes[v] + 30.0 * (n - 1 - v); };
     for (int v = t.v_lo; v <= t.v_hi; ++v) total += (double)t.count[v] * (red + t.lanes[v] * leaves(v));
