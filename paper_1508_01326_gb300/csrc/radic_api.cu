@@ -394,10 +394,11 @@ int make_plan_uncached(int m, int n, int mode, const radic_options* o, unsigned 
   // processors of a full-occupancy grid, so every processor gets one task and
   // no SM waits on a tail; an explicit ranks_per_task overrides the run length.
   if (mapping == RADIC_MAP_PREFIX) return plan_prefix(pl, d, sms, per_sm, units, p);
-  // Floating-point groups: the split is that of 512 threads per SM whatever
-  // the kernel's registers leave resident (groups of 32: 384), because the
-  // binary32 sums of bounds round per run; the blocks beyond those resident even out the tail
-  // (17 x 22: 485 us against 508 with runs for the resident blocks).
+  // Floating-point groups: the split into runs is that of 512 threads per SM
+  // whatever the kernel's registers leave resident (at 128 threads a block:
+  // four blocks for groups of 16, three for groups of 32), because the binary32
+  // sums of bounds round per run; the blocks beyond those resident even out the
+  // tail (17 x 22: 485 us against 508 with runs for the resident blocks).
   const unsigned long long cap =
       (unsigned long long)sms * (mapping == RADIC_MAP_GROUP && mode != kModeExact ? 512 / pl.threads : per_sm);
   const unsigned long long per_block =
@@ -412,6 +413,16 @@ int make_plan_uncached(int m, int n, int mode, const radic_options* o, unsigned 
   pl.tasks = (units + L - 1) / L;
   const unsigned long long need = (pl.tasks + per_block - 1) / per_block;
   unsigned long long blocks = need < cap ? need : cap;
+  // Runs of single minors: a second wave of blocks would start every
+  // elimination afresh; the resident groups take consecutive minors instead,
+  // which resume it (22 x 25: 149 us in two waves, 117 now, 113 by a kernel
+  // that left four blocks resident).  With runs of two and three minors the
+  // second wave is the better one (26 x 29 199 us against 267).
+  const unsigned long long resident = (unsigned long long)sms * per_sm;
+  if (mapping == RADIC_MAP_GROUP && blocks > resident && L == 1) {
+    const unsigned long long per = (blocks + resident - 1) / resident;
+    blocks = (need + per - 1) / per;
+  }
   if (d.blocks > 0) blocks = (unsigned long long)d.blocks;
   if (blocks < 1) blocks = 1;
   if (blocks > (1ull << 20)) return RADIC_EINVAL;

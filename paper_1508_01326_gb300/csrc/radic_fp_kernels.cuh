@@ -576,24 +576,25 @@ __global__ void __maxnreg__(G == 16 ? 128 : 168) k_fp_group(SingleArgs a) {
   unsigned long long* flist = nullptr;
   if constexpr (kMixed && !kTerms) flist = a.flag_ranks + gwarp * (unsigned long long)a.flag_cap;
 
-  for (unsigned long long base = gwarp * kSegs; base < a.tasks; base += nsegs) {
-    const unsigned long long task = base + seg;
-    const bool tact = task < a.tasks;
-    const unsigned long long q0 = qbase + (tact ? task : 0ull) * L;
-    const unsigned long long q1 = min(q0 + L, qlim);
-    int cs = 0;  // column c_sub
-    {
-      int c[G];
-      unrank_dyn<G>(q0, n, m, sm.binom, m + 1, c);
+  // Where the grid holds fewer groups than there are tasks, a group takes `per`
+  // consecutive ones and goes on with the elimination of the last; sums are
+  // closed per task all the same.
+  const unsigned long long per = (a.tasks + nsegs - 1) / nsegs, base = gwarp * kSegs * per;
+  unsigned long long q = qbase + (base + seg * per) * L;
+  const unsigned long long qend = min(q + per * L, qlim);  // q >= qend: nothing to do
+  int cs = 0;                                              // column c_sub
+  if (base < a.tasks) {
+    int c[G];
+    unrank_dyn<G>(q < qend ? q : qbase, n, m, sm.binom, m + 1, c);
 #pragma unroll
-      for (int j = 0; j < G; ++j) cs = sub == j ? c[j] : cs;
-    }
+    for (int j = 0; j < G; ++j) cs = sub == j ? c[j] : cs;
+  }
+  int first = 0;  // first column that changed since the previous minor
+  for (unsigned long long t = base; t < min(base + per, a.tasks); ++t) {
     Ff run;
     float run_abs = 0.0f, run_bnd = 0.0f;
-    int first = 0;  // first column that changed since the previous minor
-    for (unsigned long long it = 0; it < L; ++it) {
-      const unsigned long long q = q0 + it;
-      const bool act = tact && q < q1;
+    for (unsigned long long it = 0; it < L; ++it, ++q) {
+      const bool act = q < qend;
       T gmax, det;
       float b = 0.0f;
       bool bad = false;
@@ -666,7 +667,7 @@ __global__ void __maxnreg__(G == 16 ? 128 : 168) k_fp_group(SingleArgs a) {
       // successor: the last column that can still move does, the later ones follow it
       const unsigned can = (__ballot_sync(kFull, sub < m && cs < n - m + sub) >> (seg * G)) & segbits;
       const int pos = can != 0u ? 31 - __clz(can) : 0, cp = __shfl_sync(kFull, cs, pos, G);
-      const bool more = q + 1 < q1;
+      const bool more = q + 1 < qend;
       if (more && sub >= pos && sub < m) cs = cp + 1 + sub - pos;
       if constexpr (!kTerms) first = __reduce_min_sync(kFull, more ? pos : m - 1);  // over the warp's groups
     }
