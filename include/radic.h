@@ -323,8 +323,8 @@ typedef struct radic_batch_graph radic_batch_graph;
 /* Per-m tuning of the batched path (written by the autotuner; zero fields
  * mean "default").  kind[m]: RADIC_MAP_PREFIX or RADIC_MAP_THREAD (per-minor,
  * m <= 8).  task_cost[m]: target work per lane and task, in the plan's cost
- * units (default 30000 for large batches, less for small ones; smaller =
- * more, shorter tasks). */
+ * units (smaller = more, shorter tasks; default 30000, in binary64 less where
+ * the batch's whole work spread over the device's SMs is less). */
 typedef struct radic_batch_tuning {
   int32_t kind[RADIC_MAX_M + 1];
   double task_cost[RADIC_MAX_M + 1];
@@ -358,7 +358,12 @@ typedef struct radic_batch_tuning {
  * RADIC_MODE_PAIR or RADIC_MODE_FP64.  The work of every matrix is cut into warp tasks
  * (runs of prefixes or of dictionary ranks, per the tuning) for persistent
  * kernels with atomic work queues, one per tier and m, followed by a
- * per-matrix fixed-order reduction.  Limits: 1 <= m <= 10, n <= 64.
+ * per-matrix fixed-order reduction: calls with one plan give the same bits.
+ * The binary64 split follows the whole batch unless tuning->task_cost names
+ * it, so the last bits of a matrix's binary64 value and abs_sum may differ
+ * between batches that hold it (far below err_bound); with task_cost given
+ * the split, and with it every bit, depends on the matrix's shape only.  The
+ * other tiers' splits never depend on the batch.  Limits: 1 <= m <= 10, n <= 64.
  * The plan is host memory owned by the library until
  * radic_batch_plan_destroy.  Errors: RADIC_EINVAL, RADIC_EUNSUPPORTED
  * (EXACT mode, m > 10), RADIC_ECUDA. */

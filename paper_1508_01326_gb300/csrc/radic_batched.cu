@@ -87,19 +87,23 @@ double head_cost(int m, int D, int n, int v0, int v1) {
 
 // Work per lane and task, in the cost units above, when the tuning names none:
 // kTaskCost, or in binary64 about an eighth of a warp's share of the batch
-// (persistent kernels of eight warps on each of the GB300's 152 SMs) where that
+// (persistent kernels of eight warps on each SM) where that
 // is less, down to a floor below which staging the matrix again for every task
 // costs more than the balance gains: 1500, and 3000 where the matrices
 // themselves already make small or many tasks.  (Measured in binary64: 300
 // matrices, m = 2..9, n - m <= 16, 3.3 ms with kTaskCost for every batch, the
 // SMs busy 14 to 63% of the kernels' time, 1.5 ms now, 81 to 93% in the two
 // kernels with most work; 30 of 8 x (9..20) 1.28 ms, 0.23 with a floor of 3000,
-// 0.15 with 1500; 2000 with m = 2..6, n - m <= 20, 1.21 ms and 0.87 now.)
+// 0.15 with 1500; 2000 with m = 2..6, n - m <= 20, 1.21 ms and 0.87 now.)  A
+// split by shape alone, fine enough for small batches, would give large ones ten
+// times the tasks to plan and keep (4096 of 10 x 30: 38 million); a caller who
+// wants a matrix's last bits independent of its batch names the task cost.
 constexpr double kTaskCost = 30000.0;
-double default_task_cost(double total_cost, int batch) {
-  constexpr double kWarps = 152.0 * 8.0;
-  const double share = total_cost / (kWarps * 32.0), per_matrix = total_cost / (batch * 32.0);
-  const double least = (batch > kWarps || per_matrix < 500.0) ? 3000.0 : 1500.0;
+constexpr int kHostPlanSms = 152;  // host-only task lists: the GB300's SMs
+double default_task_cost(double total_cost, int batch, int sms) {
+  const double warps = sms * 8.0;
+  const double share = total_cost / (warps * 32.0), per_matrix = total_cost / (batch * 32.0);
+  const double least = (batch > warps || per_matrix < 500.0) ? 3000.0 : 1500.0;
   return std::min(kTaskCost, std::max(least, share / 8.0));
 }
 
@@ -389,9 +393,10 @@ int enqueue(const radic_batch_plan* pl, const void* A, int dtype, radic_result* 
 
 namespace {
 // Host part of the plan: routing of every matrix to a tier, its tasks, and
-// their order.  Returns a RADIC_* code; `pl` is filled on success.
+// their order, for a device of `sms` SMs.  Returns a RADIC_* code; `pl` is
+// filled on success.
 int plan_tasks(radic_batch_plan* pl, const int32_t* m, const int32_t* n, const int64_t* offsets, int batch, int mode,
-               const radic_batch_tuning* tuning) {
+               const radic_batch_tuning* tuning, int sms) {
   pl->batch = batch;
   pl->mode = mode;
   if (tuning && tuning->tol > 0.0) pl->tol = tuning->tol;
@@ -434,7 +439,7 @@ int plan_tasks(radic_batch_plan* pl, const int32_t* m, const int32_t* n, const i
     }
     cost += matrix_cost(m[b], n[b], task_kind(m[b], n[b], tier, tuning));
   }
-  const double auto_cost = default_task_cost(cost, batch);
+  const double auto_cost = default_task_cost(cost, batch, sms);
   for (int b = 0; b < batch; ++b) make_tasks(*pl, b, pl->tier[b], tuning, auto_cost);
   // per group (m, task path) and tier (binary32 before pairs), largest tasks
   // first (longest-processing-time order for each queue)
@@ -489,8 +494,9 @@ int radic_batch_plan_create(const int32_t* m, const int32_t* n, const int64_t* o
   *plan = nullptr;
   radic_batch_plan* pl = new (std::nothrow) radic_batch_plan;
   if (!pl) return RADIC_EINVAL;
+  const int sms = device_sm_count();
   {
-    const int rc = plan_tasks(pl, m, n, offsets, batch, mode, tuning);
+    const int rc = plan_tasks(pl, m, n, offsets, batch, mode, tuning, sms > 0 ? sms : kHostPlanSms);
     if (rc != RADIC_OK) {
       delete pl;
       return rc;
@@ -539,7 +545,6 @@ int radic_batch_plan_create(const int32_t* m, const int32_t* n, const int64_t* o
       if (n64[m] > 0) pl->slice64[m] = slice(m, n64[m], d64[m], ((m + 1) / 2) * 2, 8, false);
     }
   }
-  const int sms = device_sm_count();
   if (sms <= 0) {
     delete pl;
     return RADIC_ECUDA;
@@ -635,7 +640,7 @@ int radic_batch_plan_tasks_host(const int32_t* m, const int32_t* n, const int64_
   if (batch < 1 || !m || !n || !offsets || !n_tasks || capacity < 0 || (capacity > 0 && !tasks)) return RADIC_EINVAL;
   if (mode != RADIC_MODE_FP64 && mode != RADIC_MODE_MIXED) return RADIC_EUNSUPPORTED;
   radic_batch_plan pl;
-  const int rc = plan_tasks(&pl, m, n, offsets, batch, mode, tuning);
+  const int rc = plan_tasks(&pl, m, n, offsets, batch, mode, tuning, kHostPlanSms);
   if (rc != RADIC_OK) return rc;
   *n_tasks = (int64_t)(pl.t32.size() + pl.t64.size());
   int64_t i = 0;
