@@ -62,9 +62,11 @@ __device__ long long prefix_leaves_f64(const FpSmem<double>& sm, int n, int m, i
 // the flagged minors; when nothing was flagged every block returns at once.
 // Otherwise block b owns the flag lists of a contiguous range of warps of the
 // main kernel, and the last block adds the recomputed sums to the main totals
-// kept in the workspace header and rewrites the result.
+// kept in the workspace header and rewrites the result.  One block per SM, so
+// the registers are its own: left to choose, the compiler takes 64 and spills
+// 440 bytes per thread (30 x 32, every minor flagged: 7.7 ms).
 template <int MC>
-__global__ void __launch_bounds__(128) k_mixed_fixup(SingleArgs a, int main_blocks, int tier) {
+__global__ void __launch_bounds__(128, 1) k_mixed_fixup(SingleArgs a, int main_blocks, int tier) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int has_work;
   const bool overflow = __ldcg(&a.hdr->overflow) != 0;
