@@ -149,9 +149,8 @@ __device__ __forceinline__ void successor(int (&c)[M], int n) {
   }
 }
 
-// Dynamic-m form; returns the first position that changed.
 template <int G>
-__device__ __forceinline__ int successor_dyn(int (&c)[G], int n, int m) {
+__device__ __forceinline__ void successor_dyn(int (&c)[G], int n, int m) {
   int pos = 0;
 #pragma unroll
   for (int t = 0; t < G; ++t)
@@ -161,7 +160,6 @@ __device__ __forceinline__ int successor_dyn(int (&c)[G], int n, int m) {
     if (t == pos) c[t] += 1;
     if (t > 0 && t > pos && t < m) c[t] = c[t - 1] + 1;
   }
-  return pos;
 }
 
 // (-1)^(r+s) of Eq. (1): r = m(m+1)/2 and s = sum of the 1-based indices,
