@@ -107,8 +107,8 @@ enum { RADIC_MODE_FP64 = 0, RADIC_MODE_MIXED = 1, RADIC_MODE_EXACT = 2, RADIC_MO
  *            triple product).  Same pivots and elimination steps as
  *            per-minor LU, shared by the subtree.  In EXACT mode the
  *            determinant needs only the signed sum, so the units are heads
- *            of m-G columns (G = 2..6, from the plan's cost model, or an
- *            explicit prefix_depth) whose subtrees are summed by linearity
+ *            of m-G columns (G = 2..6 from the plan's cost model; an
+ *            explicit prefix_depth, 2 or 3, is taken as G) whose subtrees are summed by linearity
  *            without forming the minors; radic_terms uses depth D.
  *  AUTO   -- PREFIX when 3 <= m <= n within its limit, else THREAD when
  *            m <= 8 (12 for EXACT), else GROUP. */
