@@ -42,7 +42,7 @@
 // SM, whether or not all its lanes are used) or, in pairs, dependent binary32
 // chains at 8 warps per SM.  G trades the number of heads, C(n-G, m-G),
 // against the cost of a column (bwd_plan).  256 matrices of 6 x 28, binary64:
-// 0.60 ms with G = 4 (6.0 ms with G = 2 and lanes grouped by equal v, the pipe
+// 0.58 ms with G = 4 (6.0 ms with G = 2 and lanes grouped by equal v, the pipe
 // 83% busy; 0.57 ms with R taken forwards, see above).
 //
 // Lanes take heads in colexicographic order (by last column v, then in
@@ -846,6 +846,7 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_resident(M)) k_backward_heads
           for (int S = 1; S < FULL; ++S) at[(S - 1) * 32] = R[S];
 #pragma unroll
           for (int d = 0; d < G; ++d) at[(FULL - 1 + d) * 32] = z[d];
+          if (step > 0 && col == a0) break;  // R before the segment was kept on the way back
         }
         first_column<T, G, G, FULL>(R, z);
       }
