@@ -52,7 +52,7 @@ __host__ __device__ inline size_t fp_smem_bytes(int n, int m, int cs, int elem, 
   off += ((size_t)n * cs * elem + 15) / 16 * 16;
   off += ((size_t)m * 4 + 15) / 16 * 16;
   off += ((size_t)n * 8 + 15) / 16 * 16;
-  off += (size_t)kScratchWords * (threads / 32) * 8;
+  off += ((size_t)kScratchWords * (threads / 32) * 8 + 15) / 16 * 16;
   if (dbl) off += (size_t)n * ((m + 1) / 2 * 2) * 8;
   return off;
 }
@@ -76,7 +76,7 @@ struct FpSmem {
     colnorm = reinterpret_cast<Rad<T>*>(base + off);
     off += ((size_t)n * 8 + 15) / 16 * 16;
     scratch = reinterpret_cast<double*>(base + off);
-    off += (size_t)kScratchWords * (blockDim.x / 32) * 8;
+    off += ((size_t)kScratchWords * (blockDim.x / 32) * 8 + 15) / 16 * 16;
     As64 = std::is_same<T, ff>::value ? reinterpret_cast<double*>(base + off) : nullptr;
   }
 };
