@@ -144,7 +144,8 @@ void plan_subtree(SinglePlan& pl, const radic_options& d, int sms) {
   }
 }
 
-int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsigned long long units,
+// `launch`: the plan is for this device, not for a host-only query.
+int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsigned long long units, bool launch,
                 SinglePlan* out) {
   const int m = pl.m, n = pl.n, D = pl.depth, P = m - D;
   PrefixTable& t = pl.ptab;
@@ -288,7 +289,7 @@ int plan_prefix(SinglePlan pl, const radic_options& d, int sms, int per_sm, unsi
   pl.ranks_per_task = (units + procs - 1) / procs;
   if (pl.ranks_per_task < 1) pl.ranks_per_task = 1;
   pl.tasks = (units + pl.ranks_per_task - 1) / pl.ranks_per_task;
-  if (pl.mode == kModeExact) plan_subtree(pl, d, sms);
+  if (pl.mode == kModeExact && launch) plan_subtree(pl, d, sms);  // asks the device for its occupancy
   layout_workspace(pl);
   *out = pl;
   return RADIC_OK;
@@ -393,7 +394,7 @@ int make_plan_uncached(int m, int n, int mode, const radic_options* o, unsigned 
   // one contiguous run of about C(n,m)/K ranks.  K is the number of resident
   // processors of a full-occupancy grid, so every processor gets one task and
   // no SM waits on a tail; an explicit ranks_per_task overrides the run length.
-  if (mapping == RADIC_MAP_PREFIX) return plan_prefix(pl, d, sms, per_sm, units, p);
+  if (mapping == RADIC_MAP_PREFIX) return plan_prefix(pl, d, sms, per_sm, units, per_sm_given <= 0, p);
   // Floating-point groups: the split into runs is that of 512 threads per SM
   // whatever the kernel's registers leave resident (at 128 threads a block:
   // four blocks for groups of 16, three for groups of 32), because the binary32
