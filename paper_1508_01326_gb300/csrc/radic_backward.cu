@@ -964,7 +964,7 @@ const void* bwd_heads_kernel(int m, int G) {
 }
 
 struct BwdPlan {
-  int G = 0, chunks = 1, seg = 0;
+  int G = 0, chunks = 1;
 };
 
 // Subtree depth and blocks per matrix of the head kernel.  Estimate for every
@@ -1002,18 +1002,21 @@ BwdPlan bwd_plan(int batch, int m, int n, int sms) {
       best.chunks = (int)std::max(1ll, std::min(std::min(by_work, want), 65535ll));
     }
   }
-  // Segments as long as the shared memory of the blocks that run together on an
-  // SM allows: a segment's columns are computed twice, but for the first's.
-  // (5000 matrices of 3 x 30, 16 columns and three blocks per SM 507 us, 12 and
-  // four 449; 64 of them, one block per SM, 12 columns 51 us, 24 45.)
-  const long long blocks = (long long)batch * best.chunks;
+  return best;
+}
+
+// Columns per segment of the suffix sums: as many as the shared memory of the
+// blocks that run together on an SM allows, because a segment's columns are
+// computed twice, but for the first's.  (5000 matrices of 3 x 30, 16 columns and
+// three blocks per SM 507 us, 12 and four 449; 64 of them, one block per SM, 12
+// columns 51 us, 24 45.)
+int bwd_segment(long long blocks, int m, int n, int G, int sms) {
   const int resident = (int)std::max(1ll, std::min<long long>((blocks + sms - 1) / sms, bwd_resident(m)));
   const size_t room = std::min<size_t>(228 * 1024 / resident - 1024, 227 * 1024);
-  const int cols = n - (m - best.G);
-  best.seg = bwd_min_segment(best.G);
-  while (best.seg < cols && BwdSmem<double>(nullptr, n, m, best.G, best.seg + 2, kBwdThreads / 32).bytes <= room)
-    best.seg += 2;
-  return best;
+  const size_t warps = kBwdThreads / 32, col = warps * bwd_store_words(G) * 32 * 8;
+  const size_t fixed = BwdSmem<double>(nullptr, n, m, G, 0, (int)warps).bytes - warps * bwd_work_bytes(m, G, 0);
+  const int fit = (int)((room - fixed) / col) & ~1, all = (n - (m - G) + 1) & ~1;
+  return std::max(bwd_min_segment(G), std::min(fit, all));
 }
 
 int bwd_chunks(int batch, unsigned long long total) {
@@ -1089,11 +1092,12 @@ int radic_det_backward_mode(const double* A, int batch, int m, int n, int64_t ld
   const void* k;
   size_t smem;
   if (m >= 3) {  // shared per head
-    const BwdPlan p = bwd_plan(batch, m, n, device_sm_count());
+    const int sms = std::max(1, device_sm_count());
+    const BwdPlan p = bwd_plan(batch, m, n, sms);
     a.chunks = p.chunks;
-    a.seg = p.seg;
+    a.seg = bwd_segment((long long)batch * p.chunks, m, n, p.G, sms);
     k = (mode == RADIC_MODE_PAIR) ? bwd_heads_kernel<ff>(m, p.G) : bwd_heads_kernel<double>(m, p.G);
-    smem = BwdSmem<double>(nullptr, n, m, p.G, p.seg, kBwdThreads / 32).bytes;
+    smem = BwdSmem<double>(nullptr, n, m, p.G, a.seg, kBwdThreads / 32).bytes;
   } else {
     k = bwd_kernel(m);
     smem = bwd_smem(m, n);
