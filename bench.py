@@ -742,6 +742,7 @@ def measure_configs(R, W, torch, np, stream, flush, peaks, mats, A, minors, gold
         "value": r["minors"] / (ms / 1e3), "unit": UNIT, "ms": ms, "n_primes": r["n_primes"],
         "exact_ok": r["exact"] == int(golden_fraction("int8_12x40")),
         "mapping": f"{pinfo['mapping']}, subtrees of {pinfo['subtree_depth']} columns",
+        "rate": "nominal: C(n,m) over the time; subtrees are summed without forming their minors",
         "roofline": {"bound": "alu", "achieved": mult_rate, "unit": "T multiplies/s",
                      "peak": peaks["int32_mad_wide_tops"] if peaks else None,
                      "frac": mult_rate / peaks["int32_mad_wide_tops"] if peaks else None,
@@ -757,6 +758,7 @@ def measure_configs(R, W, torch, np, stream, flush, peaks, mats, A, minors, gold
         "value": math.comb(32, 8) / (ms / 1e3), "unit": UNIT, "ms": ms, "n_primes": wr["n_primes"],
         "bits": abs(wr["integer"]).bit_length(),
         "exact_ok": wr["value_exact"] == golden_fraction("fp64_8x32"),
+        "rate": "nominal, as int8_12x40_exact",
         "what": "radic_det_exact_wide: every prime in one launch of the exact kernel, Garner to limbs in its last block"}
 
     # differentiation 256 x 6 x 28: forward (batched binary64) and backward

@@ -424,7 +424,7 @@ __device__ __forceinline__ T group_det(T (&x)[G], int m, int sub, int seg, T& gm
 // What bounds it: shuffles (two for the pivot row's entry, one for its radius
 // per step) and the binary64 pipe, one multiply-add per step and warp however
 // few lanes are rows.  12 x 20 (126 thousand minors): 751 us with every minor
-// eliminated on its own, 393 us now (the pipe 66% busy while the SMs are, which
+// eliminated on its own, 377 us now (the pipe 68% busy while the SMs are, which
 // is 78% of the time: later minors of dictionary order change more columns).
 template <typename T, int G, bool kGrowth>
 struct GroupLu {
